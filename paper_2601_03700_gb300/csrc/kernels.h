@@ -33,34 +33,36 @@ static __device__ __forceinline__ float exit_similarity(int metric, float ns, fl
 void launch_pass_init(cudaStream_t st, int n_tok, int prompt_len, int decode, int* tok_seq, int* tok_pos,
                       int* row_tok, int* seq_len, int seq_cap, int max_pos, unsigned* err, int* ctr, int n_ctr,
                       float* sim, int n_layers, int* tok_exit);
-// xhat (optional, decoders): the embedded rows standardised (smode, seps) in bf16, [n_tok][D].
+// xhat: the embedded rows as the first layer's attention input (decoders: standardised by smode,
+// seps) in the model's type, [n_tok][D].
 void launch_embed(cudaStream_t st, int dt, const int* tokens, int n_tok, const int* tok_pos, const void* E,
                   const void* P, const float* type_emb, const float* g, const float* b, int family, int D, int V,
-                  float eps, float* X, unsigned* err, bf16* xhat, int smode, float seps);
+                  float eps, float* X, unsigned* err, void* xhat, int smode, float seps);
 void launch_standardize(cudaStream_t st, int dt, const float* X, int ldx, const int* in_rows, DevRange rows,
                         int max_rows, int D, int mode, float eps, void* out, int ld_out);
-void launch_layernorm_inplace(cudaStream_t st, float* X, DevRange rows, int max_rows, int D, const float* g,
-                              const float* b, float eps);
-// Exit decisions of the active rows.  metric: EXIT_*; Xin = the layer's input rows s_{i-1}
-// (local metric).  The exit kernels below take the same metric and aao_len: all-at-once
-// prompt exits (App. H.2) with aao_len = the prompt length (every row takes the decision of
-// its sequence's last prompt token; tok_pos gives a token's position), 0 = token level.
-void launch_exit_decide(cudaStream_t st, const float* Xout, const float* I, const float* Xin, int D, DevRange rows,
-                        int max_rows, const int* row_tok, const int* forced, int layer, int n_layers,
-                        const float* delta_p, int test, int metric, float* sim, int* flag, float* inv_norm,
+// LayerNorm with gain and shift of rows of X in place, and the result in the model's type in xt.
+void launch_layernorm_rows(cudaStream_t st, int dt, float* X, DevRange rows, int max_rows, int D, const float* g,
+                           const float* b, float eps, void* xt);
+// The exit step of a layer: test, inertia update, stable compaction, and the kept rows
+// standardised (smode, seps) as the next layer's attention input, in the model's type, in
+// xhat_next.  metric: EXIT_*; Xin = the layer's input rows s_{i-1}.  aao_len: all-at-once prompt
+// exits (App. H.2), = the prompt length (every row takes the decision of its sequence's last
+// prompt token; tok_pos gives a token's position), 0 = token level.  max_rows: the pass's row
+// bound.  launch_exit_decode: one CTA that holds every row in registers; returns false (nothing
+// launched) above 16 rows or rows that its registers do not hold (at D = 4096, above 4 rows).
+// launch_exit_rows: two launches over any number of rows (flag, inv_norm: one word per row).
+bool launch_exit_decode(cudaStream_t st, int dt, const float* Xin, const float* Xout, const float* I, int first, int D,
+                        int* ctr, int par, const int* row_tok, int* row_tok_next, const int* forced, int layer,
+                        int n_layers, const float* delta_p, int test, float* sim, int* exit_tok, int* exit_layer_out,
+                        float* Xnext, float* Inext, float* hsm_s, float* hsm_prev, float* hsm_I, int max_rows,
+                        void* xhat_next, int smode, float seps, int metric, int aao_len, const int* tok_pos,
                         unsigned* err);
-// Test + compaction + moves in one CTA for passes of at most EXIT_SMALL_MAX rows
-// (max_rows: the pass's row bound; at most 16 rows take a register-resident kernel, which
-// also writes xhat_next (if given): each kept row standardised (smode, seps) for the next
-// layer's attention input, bf16 [new row][D]).  Returns whether the register-resident
-// kernel ran (xhat_next written).
-constexpr int EXIT_SMALL_MAX = 256;
-bool launch_exit_small(cudaStream_t st, const float* Xin, const float* Xout, const float* I, int first, int D,
-                       int* ctr, int par, const int* row_tok, int* row_tok_next, const int* forced, int layer,
-                       int n_layers, const float* delta_p, int test, float* sim, int* exit_tok, int* exit_layer_out,
-                       float* Xnext, float* Inext, float* hsm_s, float* hsm_prev, float* hsm_I, int max_rows,
-                       bf16* xhat_next, int smode, float seps, int metric, int aao_len, const int* tok_pos,
-                       unsigned* err);
+void launch_exit_rows(cudaStream_t st, int dt, const float* Xin, const float* Xout, const float* I, int first, int D,
+                      int* ctr, int par, int max_rows, const int* row_tok, int* row_tok_next, const int* forced,
+                      int layer, int n_layers, const float* delta_p, int test, int metric, float* sim, int* flag,
+                      float* inv_norm, int* exit_tok, int* exit_layer_out, float* Xnext, float* Inext, float* hsm_s,
+                      float* hsm_prev, float* hsm_I, void* xhat, int smode, float seps, int aao_len,
+                      const int* tok_pos, unsigned* err);
 void launch_set_float(cudaStream_t st, float* p, float v);
 void launch_span_collect(cudaStream_t st, SpanSite* sites, int n, SpanTotal* tot, int n_cls);
 // Generation-step staging of the caller's inputs (forced NULL -> zeros) and outputs (each
@@ -70,12 +72,6 @@ void launch_stage_in(cudaStream_t st, float* d_delta, float delta, const int* to
 void launch_stage_out(cudaStream_t st, int batch, const int* dec_exit, int* exit_out, const int* dec_next,
                       int* next_out, const float* logits, float* logits_out, long long n_logits, const float* sim,
                       float* sim_out, int n_sim);
-void launch_exit_scan(cudaStream_t st, int* ctr, int in_parity, const int* flag, const int* row_tok,
-                      int* row_tok_next, int* exit_tok, int* dst, int* exit_layer_out, int layer, int aao_len,
-                      const int* tok_pos);
-void launch_exit_move(cudaStream_t st, const float* Xin, const float* Xout, const float* I, int first, int D,
-                      const int* n_rows, int max_rows, const int* dst, const float* inv_norm, float* Xnext,
-                      float* Inext, float* hsm_s, float* hsm_prev, float* hsm_I);
 void launch_final_scatter(cudaStream_t st, const float* X, int D, const int* n_rows, int max_rows, const int* row_tok,
                           float* final_, int* exit_layer_out, int n_layers);
 // launch_final_scatter that also writes each row standardised for the output head (hmode, heps)

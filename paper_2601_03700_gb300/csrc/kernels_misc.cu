@@ -1,5 +1,4 @@
-// Row-wise kernels of the early-exit pass: embedding, norms, the exit test with
-// active-token compaction, the HSM's non-GEMM steps, argmax, skipped-layer-fill
+// Row-wise kernels of the early-exit pass: embedding, the exit step of generation steps, the HSM's non-GEMM steps, argmax, skipped-layer-fill
 // bucketing and load-time weight repacking.
 #define ADEPT_TU_ID 3
 #include "common.cuh"
@@ -49,12 +48,12 @@ __global__ void pass_init_kernel(int n_tok, int prompt_len, int decode, int* tok
 // ---------------------------------------------------------------------------
 // embedding (s_0): token embedding (+ learned position) (+ type and LayerNorm for BERT)
 // ---------------------------------------------------------------------------
-// xhat (optional, decoders): each embedded row standardised for the first layer's
-// attention input (smode, seps), as the standardisation kernel computes it, in bf16.
+// xhat: each embedded row as the first layer's attention input, in the model's type: decoders
+// standardised (smode, seps) as the standardisation kernel computes it, the encoder as it is.
 template <typename T>
 __global__ void embed_kernel(const int* tokens, int n_tok, const int* tok_pos, const T* E, const T* P,
                              const float* type_emb, const float* g, const float* b, int family, int D, int V,
-                             float eps, float* X, unsigned* err, bf16* xhat, int smode, float seps) {
+                             float eps, float* X, unsigned* err, T* xhat, int smode, float seps) {
   PDL_ENTRY();
   __shared__ float red[32];
   const int t = blockIdx.x;
@@ -75,7 +74,6 @@ __global__ void embed_kernel(const int* tokens, int n_tok, const int* tok_pos, c
     s1 += v;
   }
   if (family != 2) {
-    if (!xhat) return;
     // the thread re-reads only the elements it wrote
     const float mu = smode == NORM_LN ? block_sum(s1, red) / D : 0.f;
     float s2 = 0.f;
@@ -86,7 +84,7 @@ __global__ void embed_kernel(const int* tokens, int n_tok, const int* tok_pos, c
     const float tot = block_sum(s2, red);
     const float rs = smode == NORM_COPY ? 1.f : rsqrtf(tot / D + seps);
     const float m0 = smode == NORM_COPY ? 0.f : mu;
-    for (int d = threadIdx.x; d < D; d += blockDim.x) xhat[(size_t)t * D + d] = __float2bfloat16_rn((x[d] - m0) * rs);
+    for (int d = threadIdx.x; d < D; d += blockDim.x) xhat[(size_t)t * D + d] = from_f<T>((x[d] - m0) * rs);
     return;
   }
   const float mu = block_sum(s1, red) / D;
@@ -96,7 +94,11 @@ __global__ void embed_kernel(const int* tokens, int n_tok, const int* tok_pos, c
     s2 += c * c;
   }
   const float rstd = rsqrtf(block_sum(s2, red) / D + eps);
-  for (int d = threadIdx.x; d < D; d += blockDim.x) x[d] = (x[d] - mu) * rstd * g[d] + b[d];
+  for (int d = threadIdx.x; d < D; d += blockDim.x) {
+    const float y = (x[d] - mu) * rstd * g[d] + b[d];
+    x[d] = y;
+    xhat[(size_t)t * D + d] = from_f<T>(y);
+  }
 }
 
 // Grid of the row kernels whose live row count is a device value, usually far below its
@@ -115,316 +117,30 @@ static int row_grid(int max_rows, int per_sm) {
 }
 static int hsm_grid(int max_rows) { return row_grid(max_rows, 2); }
 
-// ---------------------------------------------------------------------------
-// standardisation of a layer input (gains folded into the next GEMM)
-// ---------------------------------------------------------------------------
-template <typename T>
-__global__ void standardize_kernel(const float* X, int ldx, const int* in_rows, DevRange rows, int D, int mode,
-                                   float eps, T* out, int ld_out) {
-  PDL_ENTRY();
-  __shared__ float red[32];
-  const int rb = rows.b(), re = rows.e();
-  for (int r = rb + blockIdx.x; r < re; r += gridDim.x) {   // rows of the live range, in turn
-  const int src = in_rows ? in_rows[r] : r;
-  const float* x = X + (size_t)src * ldx;
-  T* o = out + (size_t)r * ld_out;
-  if (mode == NORM_COPY) {
-    for (int d = threadIdx.x; d < D; d += blockDim.x) o[d] = from_f<T>(x[d]);
-    continue;
-  }
-  float mu = 0.f;
-  if (mode == NORM_LN) {
-    float s = 0.f;
-    for (int d = threadIdx.x; d < D; d += blockDim.x) s += x[d];
-    mu = block_sum(s, red) / D;
-  }
-  float s2 = 0.f;
-  for (int d = threadIdx.x; d < D; d += blockDim.x) {
-    const float c = x[d] - mu;
-    s2 += c * c;
-  }
-  const float rstd = rsqrtf(block_sum(s2, red) / D + eps);
-  for (int d = threadIdx.x; d < D; d += blockDim.x) o[d] = from_f<T>((x[d] - mu) * rstd);
-  }
-}
-
-// In-place LayerNorm with gain and shift (the post-LN encoder's residual stream).
-__global__ void layernorm_inplace_kernel(float* X, DevRange rows, int D, const float* g, const float* b, float eps) {
-  PDL_ENTRY();
-  __shared__ float red[32];
-  const int r = rows.b() + blockIdx.x;
-  if (r >= rows.e()) return;
-  float* x = X + (size_t)r * D;
-  float s = 0.f;
-  for (int d = threadIdx.x; d < D; d += blockDim.x) s += x[d];
-  const float mu = block_sum(s, red) / D;
-  float s2 = 0.f;
-  for (int d = threadIdx.x; d < D; d += blockDim.x) {
-    const float c = x[d] - mu;
-    s2 += c * c;
-  }
-  const float rstd = rsqrtf(block_sum(s2, red) / D + eps);
-  for (int d = threadIdx.x; d < D; d += blockDim.x) x[d] = (x[d] - mu) * rstd * g[d] + b[d];
-}
-
-// ---------------------------------------------------------------------------
-// exit test (Sec. 4.1): c = <s_i, I> / (|s_i| |I|) vs delta, or the forced layer
-// ---------------------------------------------------------------------------
-
-__global__ void exit_decide_kernel(const float* Xout, const float* I, const float* Xin, int D, DevRange rows,
-                                   const int* row_tok, const int* forced, int layer, int n_layers,
-                                   const float* delta_p, int test, int metric, float* sim, int* flag,
-                                   float* inv_norm, unsigned* err) {
-  PDL_ENTRY();
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  const int r = warp;
-  if (r >= rows.e()) return;
-  const float* s = Xout + (size_t)r * D;
-  const float* in = I + (size_t)r * D;
-  const float* sp = Xin + (size_t)r * D;
-  float ns = 0.f, ni = 0.f, dot = 0.f, np_ = 0.f, dp = 0.f;
-  for (int d = lane; d < D; d += 32) {
-    const float a = s[d], c = in[d];
-    ns += a * a;
-    ni += c * c;
-    dot += a * c;
-    if (metric != EXIT_GLOBAL) {
-      const float b = sp[d];
-      np_ += b * b;
-      dp += a * b;
-    }
-  }
-  ns = warp_sum(ns);
-  ni = warp_sum(ni);
-  dot = warp_sum(dot);
-  np_ = warp_sum(np_);
-  dp = warp_sum(dp);
-  if (lane != 0) return;
-  const int tok = row_tok[r];
-  int ex = 0;
-  if (test) {
-    const float c = exit_similarity(metric, ns, ni, dot, np_, dp);
-    if (sim) sim[(size_t)tok * n_layers + (layer - 1)] = c;
-    const int f = forced ? forced[tok] : 0;
-    if (f != 0 && (f < 2 || f > n_layers)) atomicOr(err, ERRW_FORCED);
-    ex = (f > 0) ? (f == layer) : (c >= *delta_p);
-  }
-  flag[r] = ex;
-  inv_norm[r] = ns > 0.f ? rsqrtf(ns) : 0.f;
-}
-
-// Single-CTA stable compaction of the active rows: survivors keep their order in the
-// next active list; exits are appended to the pass's exit list.  Counter layout:
-// ctr[CTR_ACTIVE + parity] active counts, ctr[CTR_EXITED] exits so far,
-// ctr[CTR_PREFIX + i] exits after layer i.
-__global__ void exit_scan_kernel(int* ctr, int in_parity, const int* flag, const int* row_tok, int* row_tok_next,
-                                 int* exit_tok, int* dst, int* exit_layer_out, int layer, int aao_len,
-                                 const int* tok_pos) {
-  PDL_ENTRY();
-  __shared__ int s_stay[1024];
-  __shared__ int s_exit[1024];
-  const int n = ctr[CTR_ACTIVE + in_parity];
-  const int base = ctr[CTR_EXITED];
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int per = (n + nt - 1) / nt;
-  const int lo = min(n, tid * per), hi = min(n, lo + per);
-  // all-at-once (aao_len = prompt length): a row takes the decision of its sequence's last
-  // prompt token, which is active with it at the same row offset (sequences stay whole)
-  auto fl = [&](int r) {
-    return aao_len ? flag[min(n - 1, r + (aao_len - 1 - tok_pos[row_tok[r]]))] : flag[r];
-  };
-  int ce = 0;
-  for (int r = lo; r < hi; ++r) ce += fl(r);
-  s_exit[tid] = ce;
-  s_stay[tid] = (hi - lo) - ce;
-  __syncthreads();
-  for (int off = 1; off < nt; off <<= 1) {
-    int a = 0, b = 0;
-    if (tid >= off) {
-      a = s_exit[tid - off];
-      b = s_stay[tid - off];
-    }
-    __syncthreads();
-    s_exit[tid] += a;
-    s_stay[tid] += b;
-    __syncthreads();
-  }
-  int e = s_exit[tid] - ce;
-  int s = s_stay[tid] - ((hi - lo) - ce);
-  for (int r = lo; r < hi; ++r) {
-    const int tok = row_tok[r];
-    if (fl(r)) {
-      dst[r] = -1 - (base + e);
-      exit_tok[base + e] = tok;
-      if (exit_layer_out) exit_layer_out[tok] = layer;
-      ++e;
-    } else {
-      dst[r] = s;
-      row_tok_next[s] = tok;
-      ++s;
-    }
-  }
-  if (tid == nt - 1) {
-    const int E = s_exit[nt - 1];
-    ctr[CTR_ACTIVE + (in_parity ^ 1)] = s_stay[nt - 1];
-    ctr[CTR_EXITED] = base + E;
-    ctr[CTR_PREFIX + layer] = base + E;
-  }
-}
-
-// Moves each active row to its new place: survivors -> next layer input (s_i) and the
-// inertia with s_hat_i added (Sec. 4.1, after the test); exits -> the HSM input slots
-// (s_i, s_{i-1}, inertia before s_hat_i).  first != 0 (layer 1): the inertia starts
-// as s_hat_1 (the sum over earlier layers is empty).
-__global__ void exit_move_kernel(const float* Xin, const float* Xout, const float* I, int first, int D,
-                                 const int* n_rows, const int* dst, const float* inv_norm, float* Xnext, float* Inext,
-                                 float* hsm_s, float* hsm_prev, float* hsm_I) {
-  PDL_ENTRY();
-  const int n = *n_rows;
-  for (int r = blockIdx.x; r < n; r += gridDim.x) {
-  const int d0 = dst[r];
-  const float* s = Xout + (size_t)r * D;
-  const float* in = I + (size_t)r * D;
-  if (d0 >= 0) {
-    const float w = inv_norm[r];
-    float* xn = Xnext + (size_t)d0 * D;
-    float* inn = Inext + (size_t)d0 * D;
-    for (int d = threadIdx.x; d < D; d += blockDim.x) {
-      const float v = s[d];
-      xn[d] = v;
-      inn[d] = (first ? 0.f : in[d]) + v * w;
-    }
-  } else {
-    const size_t k = (size_t)(-1 - d0);
-    const float* sp = Xin + (size_t)r * D;
-    for (int d = threadIdx.x; d < D; d += blockDim.x) {
-      hsm_s[k * D + d] = s[d];
-      hsm_prev[k * D + d] = sp[d];
-      hsm_I[k * D + d] = in[d];
-    }
-  }
-  }
-}
-
-// The three steps above in one CTA, for passes with at most EXIT_SMALL_MAX active rows
-// (generation steps): the similarity test, the stable compaction and the row moves.
-__global__ void __launch_bounds__(256) exit_small_kernel(const float* Xin, const float* Xout, const float* I,
-                                                         int first, int D, int* ctr, int par, const int* row_tok,
-                                                         int* row_tok_next, const int* forced, int layer,
-                                                         int n_layers, const float* delta_p, int test, float* sim,
-                                                         int* exit_tok, int* exit_layer_out, float* Xnext,
-                                                         float* Inext, float* hsm_s, float* hsm_prev, float* hsm_I,
-                                                         int metric, int aao_len, const int* tok_pos,
-                                                         unsigned* err) {
-  PDL_ENTRY();
-  __shared__ int s_dst[EXIT_SMALL_MAX];
-  __shared__ float s_w[EXIT_SMALL_MAX];
-  const int n = min(ctr[CTR_ACTIVE + par], EXIT_SMALL_MAX);
-  const int base = ctr[CTR_EXITED];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  const float delta = *delta_p;
-  for (int r = warp; r < n; r += nw) {
-    const float* s = Xout + (size_t)r * D;
-    const float* in = I + (size_t)r * D;
-    const float* sp = Xin + (size_t)r * D;
-    float ns = 0.f, ni = 0.f, dot = 0.f, np_ = 0.f, dp = 0.f;
-    for (int d = lane; d < D; d += 32) {
-      const float a = s[d], c = in[d];
-      ns += a * a;
-      ni += c * c;
-      dot += a * c;
-      if (metric != EXIT_GLOBAL) {
-        const float b = sp[d];
-        np_ += b * b;
-        dp += a * b;
-      }
-    }
-    ns = warp_sum(ns);
-    ni = warp_sum(ni);
-    dot = warp_sum(dot);
-    np_ = warp_sum(np_);
-    dp = warp_sum(dp);
-    if (lane == 0) {
-      const int tok = row_tok[r];
-      int ex = 0;
-      if (test) {
-        const float c = exit_similarity(metric, ns, ni, dot, np_, dp);
-        if (sim) sim[(size_t)tok * n_layers + (layer - 1)] = c;
-        const int f = forced ? forced[tok] : 0;
-        if (f != 0 && (f < 2 || f > n_layers)) atomicOr(err, ERRW_FORCED);
-        ex = (f > 0) ? (f == layer) : (c >= delta);
-      }
-      s_dst[r] = ex;
-      s_w[r] = ns > 0.f ? rsqrtf(ns) : 0.f;
-    }
-  }
-  __syncthreads();
-  KT_MARK(0);
-  if (threadIdx.x == 0) {
-    int e = 0, k = 0;
-    for (int r = 0; r < n; ++r) {
-      const int tok = row_tok[r];
-      // all-at-once: the decision of the sequence's last prompt token, a later row not yet
-      // rewritten by this loop
-      const int rl = aao_len ? min(n - 1, r + (aao_len - 1 - tok_pos[tok])) : r;
-      if (s_dst[rl]) {
-        s_dst[r] = -1 - (base + e);
-        exit_tok[base + e] = tok;
-        if (exit_layer_out) exit_layer_out[tok] = layer;
-        ++e;
-      } else {
-        s_dst[r] = k;
-        row_tok_next[k] = tok;
-        ++k;
-      }
-    }
-    ctr[CTR_ACTIVE + (par ^ 1)] = k;
-    ctr[CTR_EXITED] = base + e;
-    ctr[CTR_PREFIX + layer] = base + e;
-  }
-  __syncthreads();
-  KT_MARK(1);
-  for (int r = warp; r < n; r += nw) {
-    const int d0 = s_dst[r];
-    const float* s = Xout + (size_t)r * D;
-    const float* in = I + (size_t)r * D;
-    if (d0 >= 0) {
-      const float w = s_w[r];
-      float* xn = Xnext + (size_t)d0 * D;
-      float* inn = Inext + (size_t)d0 * D;
-      for (int d = lane; d < D; d += 32) {
-        const float v = s[d];
-        xn[d] = v;
-        inn[d] = (first ? 0.f : in[d]) + v * w;
-      }
-    } else {
-      const size_t kk = (size_t)(-1 - d0);
-      const float* sp = Xin + (size_t)r * D;
-      for (int d = lane; d < D; d += 32) {
-        hsm_s[kk * D + d] = s[d];
-        hsm_prev[kk * D + d] = sp[d];
-        hsm_I[kk * D + d] = in[d];
-      }
-    }
-  }
-}
-
-// The same test, compaction and moves for a generation step of at most 16 rows, in one
+// The exit test, compaction and moves (see exit_rows) of a pass of at most 16 rows in one CTA and one
 // pass over memory: each row's s_i, inertia and s_{i-1} are read once into registers (a
 // row per 512 >> rshift threads), the decision and compaction run on the reduced sums,
 // and the moves are written from the registers.
+__device__ __forceinline__ void put_row4(float* o, int v, float4 a) { reinterpret_cast<float4*>(o)[v] = a; }
+__device__ __forceinline__ void put_row4(bf16* o, int v, float4 a) {
+  const __nv_bfloat162 lo = __floats2bfloat162_rn(a.x, a.y), hi = __floats2bfloat162_rn(a.z, a.w);
+  uint2 u;
+  u.x = *reinterpret_cast<const uint32_t*>(&lo);
+  u.y = *reinterpret_cast<const uint32_t*>(&hi);
+  reinterpret_cast<uint2*>(o)[v] = u;
+}
 constexpr int EXD_THREADS = 512;
 constexpr int EXD_V = 4;   // most float4 per thread per row vector
 // V: float4 per thread per row vector, the fewest that cover a row (the kernel runs cold in
 // every layer of a generation step, so its unrolled code is kept to what the rows need)
-template <int V>
+template <int V, typename T>
 __global__ void __launch_bounds__(EXD_THREADS)
     exit_decode_kernel(const float* __restrict__ Xin, const float* __restrict__ Xout, const float* __restrict__ I,
                        int first, int D, int* ctr, int par, const int* row_tok, int* row_tok_next, const int* forced,
                        int layer, int n_layers, const float* delta_p, int test, float* sim, int* exit_tok,
                        int* exit_layer_out, float* __restrict__ Xnext, float* __restrict__ Inext,
                        float* __restrict__ hsm_s, float* __restrict__ hsm_prev, float* __restrict__ hsm_I, int rshift,
-                       int max_rows, bf16* xhat_next, int smode, float seps, int metric, int aao_len,
+                       int max_rows, T* xhat_next, int smode, float seps, int metric, int aao_len,
                        const int* tok_pos, unsigned* err) {
   // Before the grid-dependency wait: everything the previous layer's exit kernel wrote (the
   // counters, the row map, the inertia and the layer input s_{i-1}), which has completed by the
@@ -549,10 +265,10 @@ __global__ void __launch_bounds__(EXD_THREADS)
     ctr[CTR_PREFIX + layer] = base + e;
   }
   __syncthreads();
-  if (xhat_next) {
+  {
     // the kept rows standardised for the next layer's attention input, as the
     // standardisation kernel computes them (two-pass: the centred second moment from the
-    // registers); written to row d0 of xhat_next in bf16
+    // registers); written to row d0 of xhat_next
     const float mu = row < n ? s_mu[row] : 0.f;
     float c2 = 0.f;
     if (row < n) {
@@ -571,18 +287,13 @@ __global__ void __launch_bounds__(EXD_THREADS)
       for (int w = row * wpr; w < (row + 1) * wpr; ++w) t += s_red[w][0];
       const float rs = smode == NORM_COPY ? 1.f : rsqrtf(t / D + seps);
       const float m0 = smode == NORM_COPY ? 0.f : mu;
-      uint2* o = reinterpret_cast<uint2*>(xhat_next + (size_t)s_dst[row] * D);
+      T* o = xhat_next + (size_t)s_dst[row] * D;
 #pragma unroll
       for (int j = 0; j < V; ++j) {
         const int v = sub + j * tpr;
         if (v < D4) {
           const float4 a = xs[j];
-          const __nv_bfloat162 lo = __floats2bfloat162_rn((a.x - m0) * rs, (a.y - m0) * rs);
-          const __nv_bfloat162 hi = __floats2bfloat162_rn((a.z - m0) * rs, (a.w - m0) * rs);
-          uint2 u;
-          u.x = *reinterpret_cast<const uint32_t*>(&lo);
-          u.y = *reinterpret_cast<const uint32_t*>(&hi);
-          o[v] = u;
+          put_row4(o, v, make_float4((a.x - m0) * rs, (a.y - m0) * rs, (a.z - m0) * rs, (a.w - m0) * rs));
         }
       }
     }
@@ -619,27 +330,29 @@ __global__ void __launch_bounds__(EXD_THREADS)
   }
 }
 
-bool launch_exit_small(cudaStream_t st, const float* Xin, const float* Xout, const float* I, int first, int D,
-                       int* ctr, int par, const int* row_tok, int* row_tok_next, const int* forced, int layer,
-                       int n_layers, const float* delta_p, int test, float* sim, int* exit_tok, int* exit_layer_out,
-                       float* Xnext, float* Inext, float* hsm_s, float* hsm_prev, float* hsm_I, int max_rows,
-                       bf16* xhat_next, int smode, float seps, int metric, int aao_len, const int* tok_pos,
-                       unsigned* err) {
+bool launch_exit_decode(cudaStream_t st, int dt, const float* Xin, const float* Xout, const float* I, int first, int D,
+                        int* ctr, int par, const int* row_tok, int* row_tok_next, const int* forced, int layer,
+                        int n_layers, const float* delta_p, int test, float* sim, int* exit_tok, int* exit_layer_out,
+                        float* Xnext, float* Inext, float* hsm_s, float* hsm_prev, float* hsm_I, int max_rows,
+                        void* xhat_next, int smode, float seps, int metric, int aao_len, const int* tok_pos,
+                        unsigned* err) {
   int rshift = 0;
   while ((1 << rshift) < max_rows) ++rshift;
-  const bool aligned = ((uintptr_t)Xin | (uintptr_t)Xout | (uintptr_t)I | (uintptr_t)Xnext | (uintptr_t)Inext |
-                        (uintptr_t)hsm_s | (uintptr_t)hsm_prev | (uintptr_t)hsm_I) % 16 == 0;
-  if (max_rows <= 16 && D % 4 == 0 && D / 4 <= EXD_V * (EXD_THREADS >> rshift) && aligned) {
-    auto* kern = D / 4 <= 2 * (EXD_THREADS >> rshift) ? exit_decode_kernel<2> : exit_decode_kernel<EXD_V>;
-    launch_k(kern, 1, EXD_THREADS, 0, st, Xin, Xout, I, first, D, ctr, par, row_tok, row_tok_next, forced,
-             layer, n_layers, delta_p, test, sim, exit_tok, exit_layer_out, Xnext, Inext, hsm_s, hsm_prev, hsm_I,
-             rshift, max_rows, xhat_next, smode, seps, metric, aao_len, tok_pos, err);
-    return true;
+  if (max_rows > 16 || D / 4 > EXD_V * (EXD_THREADS >> rshift)) return false;
+  const bool small = D / 4 <= 2 * (EXD_THREADS >> rshift);
+#define GO(V, T)                                                                                                     \
+  launch_k(exit_decode_kernel<V, T>, 1, EXD_THREADS, 0, st, Xin, Xout, I, first, D, ctr, par, row_tok, row_tok_next, \
+           forced, layer, n_layers, delta_p, test, sim, exit_tok, exit_layer_out, Xnext, Inext, hsm_s, hsm_prev,     \
+           hsm_I, rshift, max_rows, (T*)xhat_next, smode, seps, metric, aao_len, tok_pos, err)
+  if (dt == 1) {
+    if (small) GO(2, bf16);
+    else GO(EXD_V, bf16);
+  } else {
+    if (small) GO(2, float);
+    else GO(EXD_V, float);
   }
-  launch_k(exit_small_kernel, 1, 256, 0, st, Xin, Xout, I, first, D, ctr, par, row_tok, row_tok_next, forced, layer,
-           n_layers, delta_p, test, sim, exit_tok, exit_layer_out, Xnext, Inext, hsm_s, hsm_prev, hsm_I, metric,
-           aao_len, tok_pos, err);
-  return false;
+#undef GO
+  return true;
 }
 
 __global__ void set_float_kernel(float* p, float v) {
@@ -774,7 +487,7 @@ template <typename T, int EPT>
 __global__ void __launch_bounds__(256) embed_reg_kernel(const int* tokens, int n_tok, const int* tok_pos, const T* E,
                                                         const T* P, const float* type_emb, const float* g,
                                                         const float* b, int family, int D, int V, float eps, float* X,
-                                                        unsigned* err, bf16* xhat, int smode, float seps) {
+                                                        unsigned* err, T* xhat, int smode, float seps) {
   PDL_ENTRY();
   __shared__ float red[32];
   const int t = blockIdx.x;
@@ -808,7 +521,6 @@ __global__ void __launch_bounds__(256) embed_reg_kernel(const int* tokens, int n
       const int d = threadIdx.x + j * blockDim.x;
       if (d < D) x[d] = v[j];
     }
-    if (!xhat) return;
   }
   float mu = 0.f;
   if (ln) {
@@ -829,7 +541,7 @@ __global__ void __launch_bounds__(256) embed_reg_kernel(const int* tokens, int n
 #pragma unroll
     for (int j = 0; j < EPT; ++j) {
       const int d = threadIdx.x + j * blockDim.x;
-      if (d < D) xhat[(size_t)t * D + d] = __float2bfloat16_rn((v[j] - m0) * rs);
+      if (d < D) xhat[(size_t)t * D + d] = from_f<T>((v[j] - m0) * rs);
     }
     return;
   }
@@ -837,7 +549,11 @@ __global__ void __launch_bounds__(256) embed_reg_kernel(const int* tokens, int n
 #pragma unroll
   for (int j = 0; j < EPT; ++j) {
     const int d = threadIdx.x + j * blockDim.x;
-    if (d < D) x[d] = (v[j] - mu) * rstd * g[d] + b[d];
+    if (d < D) {
+      const float y = (v[j] - mu) * rstd * g[d] + b[d];
+      x[d] = y;
+      xhat[(size_t)t * D + d] = from_f<T>(y);
+    }
   }
 }
 
@@ -1416,11 +1132,11 @@ void launch_pass_init(cudaStream_t st, int n_tok, int prompt_len, int decode, in
 
 void launch_embed(cudaStream_t st, int dt, const int* tokens, int n_tok, const int* tok_pos, const void* E,
                   const void* P, const float* type_emb, const float* g, const float* b, int family, int D, int V,
-                  float eps, float* X, unsigned* err, bf16* xhat, int smode, float seps) {
+                  float eps, float* X, unsigned* err, void* xhat, int smode, float seps) {
   if (D <= 16 * 256) {
 #define EMB(T, EPT)                                                                                                  \
   launch_k(embed_reg_kernel<T, EPT>, n_tok, 256, 0, st, tokens, n_tok, tok_pos, (const T*)E, (const T*)P, type_emb, g, \
-           b, family, D, V, eps, X, err, xhat, smode, seps)
+           b, family, D, V, eps, X, err, (T*)xhat, smode, seps)
     if (dt == 1) {
       if (D <= 4 * 256) EMB(bf16, 4);
       else EMB(bf16, 16);
@@ -1433,49 +1149,10 @@ void launch_embed(cudaStream_t st, int dt, const int* tokens, int n_tok, const i
   }
   if (dt == 1)
     launch_k(embed_kernel<bf16>, n_tok, 256, 0, st, tokens, n_tok, tok_pos, (const bf16*)E, (const bf16*)P, type_emb, g,
-             b, family, D, V, eps, X, err, xhat, smode, seps);
+             b, family, D, V, eps, X, err, (bf16*)xhat, smode, seps);
   else
     launch_k(embed_kernel<float>, n_tok, 256, 0, st, tokens, n_tok, tok_pos, (const float*)E, (const float*)P, type_emb,
-             g, b, family, D, V, eps, X, err, xhat, smode, seps);
-}
-
-void launch_standardize(cudaStream_t st, int dt, const float* X, int ldx, const int* in_rows, DevRange rows,
-                        int max_rows, int D, int mode, float eps, void* out, int ld_out) {
-  if (max_rows <= 0) return;
-  if (dt == 1)
-    launch_k(standardize_kernel<bf16>, row_grid(max_rows, 8), 256, 0, st, X, ldx, in_rows, rows, D, mode, eps, (bf16*)out, ld_out);
-  else
-    launch_k(standardize_kernel<float>, row_grid(max_rows, 8), 256, 0, st, X, ldx, in_rows, rows, D, mode, eps, (float*)out, ld_out);
-}
-
-void launch_layernorm_inplace(cudaStream_t st, float* X, DevRange rows, int max_rows, int D, const float* g,
-                              const float* b, float eps) {
-  if (max_rows <= 0) return;
-  launch_k(layernorm_inplace_kernel, max_rows, 256, 0, st, X, rows, D, g, b, eps);
-}
-
-void launch_exit_decide(cudaStream_t st, const float* Xout, const float* I, const float* Xin, int D, DevRange rows,
-                        int max_rows, const int* row_tok, const int* forced, int layer, int n_layers,
-                        const float* delta_p, int test, int metric, float* sim, int* flag, float* inv_norm,
-                        unsigned* err) {
-  if (max_rows <= 0) return;
-  launch_k(exit_decide_kernel, cdiv(max_rows, 8), 256, 0, st, Xout, I, Xin, D, rows, row_tok, forced, layer, n_layers,
-           delta_p, test, metric, sim, flag, inv_norm, err);
-}
-
-void launch_exit_scan(cudaStream_t st, int* ctr, int in_parity, const int* flag, const int* row_tok,
-                      int* row_tok_next, int* exit_tok, int* dst, int* exit_layer_out, int layer, int aao_len,
-                      const int* tok_pos) {
-  launch_k(exit_scan_kernel, 1, 1024, 0, st, ctr, in_parity, flag, row_tok, row_tok_next, exit_tok, dst, exit_layer_out,
-           layer, aao_len, tok_pos);
-}
-
-void launch_exit_move(cudaStream_t st, const float* Xin, const float* Xout, const float* I, int first, int D,
-                      const int* n_rows, int max_rows, const int* dst, const float* inv_norm, float* Xnext,
-                      float* Inext, float* hsm_s, float* hsm_prev, float* hsm_I) {
-  if (max_rows <= 0) return;
-  launch_k(exit_move_kernel, row_grid(max_rows, 8), 256, 0, st, Xin, Xout, I, first, D, n_rows, dst, inv_norm, Xnext, Inext, hsm_s,
-                                             hsm_prev, hsm_I);
+             g, b, family, D, V, eps, X, err, (float*)xhat, smode, seps);
 }
 
 void launch_final_scatter(cudaStream_t st, const float* X, int D, const int* n_rows, int max_rows, const int* row_tok,

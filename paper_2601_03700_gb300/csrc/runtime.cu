@@ -1050,14 +1050,14 @@ static adept_status run_pass(adept_model* m, int n_tok, int batch, int prompt_le
   launch_pass_init(st, n_tok, prompt_len, decode ? 1 : 0, m->tok_seq, m->tok_pos, m->row_tok[0], m->d_seq_len,
                    m->max_blocks_per_seq * c.kv_block_tokens, fam == ADEPT_FAMILY_LLAMA ? 0 : c.max_pos,
                    m->err_word, m->ctr, ctr_words(N), sim_out, N, stop ? m->tok_exit : nullptr);
-  // passes of at most DG_MAX_M rows (bf16 decoders): the producer of each layer's input
-  // (the embedding, then the exit kernel) also writes it standardised into xn, and the O
-  // projection hands the tile statistics of its output to the FFN input's GEMM
+  // the producer of each layer's input (the embedding, then the exit step) also writes it as the
+  // attention input (standardised, in the model's type) into xn; in passes of at most DG_MAX_M
+  // rows (bf16 decoders) the O projection hands the tile statistics of its output to the FFN
+  // input's GEMM
   const bool dgrows = n_tok <= DG_MAX_M && m->dt == ADEPT_DTYPE_BF16 && m->use_dg && !m->force_simt &&
                       fam != ADEPT_FAMILY_BERT;
   launch_embed(st, m->dt, tokens, n_tok, m->tok_pos, m->tok_emb, m->pos_emb, m->type_emb, m->emb_g, m->emb_b, fam, D,
-               m->V, eps, m->X_in[0], m->err_word, dgrows ? (bf16*)m->xn : nullptr, amode, eps);
-  bool xn_valid = dgrows;   // xn holds X_in[par] standardised
+               m->V, eps, m->X_in[0], m->err_word, m->xn, amode, eps);
   m->launches += 2;
   const KVCacheView cv = cache_view(m);
   const int causal = fam != ADEPT_FAMILY_BERT;
@@ -1078,6 +1078,23 @@ static adept_status run_pass(adept_model* m, int n_tok, int batch, int prompt_le
     float* Ii;
     int* rt;
   } pend = {false, 0, 0, nullptr, nullptr, nullptr};
+  // the exit step of layer `layer` on its own: one CTA that holds the rows where it can, else two
+  // launches over the rows
+  auto exit_step = [&](int layer, int p, float* Xi, float* Ii, int* rt) {
+    const int test = layer >= 2;
+    if (launch_exit_decode(st, m->dt, Xi, m->X_out, Ii, layer == 1, D, m->ctr, p, rt, m->row_tok[p ^ 1], forced, layer,
+                           N, m->d_delta, test, sim_out, m->exit_tok, exit_w, m->X_in[p ^ 1], m->I[p ^ 1], m->hsm_s,
+                           m->hsm_prev, m->hsm_I, n_tok, m->xn, amode, eps, m->exit_metric, aao_len, m->tok_pos,
+                           m->err_word)) {
+      m->launches += 1;
+      return;
+    }
+    launch_exit_rows(st, m->dt, Xi, m->X_out, Ii, layer == 1, D, m->ctr, p, n_tok, rt, m->row_tok[p ^ 1], forced, layer,
+                     N, m->d_delta, test, m->exit_metric, sim_out, m->flag, m->inv_norm, m->exit_tok, exit_w,
+                     m->X_in[p ^ 1], m->I[p ^ 1], m->hsm_s, m->hsm_prev, m->hsm_I, m->xn, amode, eps, aao_len,
+                     m->tok_pos, m->err_word);
+    m->launches += 2;
+  };
   int par = 0;
   for (int i = 1; i <= N; ++i) {
     const int l0 = i - 1;
@@ -1099,12 +1116,10 @@ static adept_status run_pass(adept_model* m, int n_tok, int batch, int prompt_le
     pr[0].epi.row_tok = rt; pr[0].epi.tok_seq = m->tok_seq; pr[0].epi.tok_pos = m->tok_pos;
     pr[0].epi.cache = cv; pr[0].epi.layer0 = l0; pr[0].epi.n_q_cols = Dq; pr[0].epi.n_kv_cols = Dkv;
     pr[0].epi.head_dim = m->dh; pr[0].epi.rope = fam == ADEPT_FAMILY_LLAMA; pr[0].epi.rope_table = m->rope_table;
-    // attention input: standardised (gain folded into W_qkv)
+    // attention input: xn, standardised (gain folded into W_qkv)
     if (!decode && i >= 3 && !stop) {
       pr[1] = kv_problem(m, l0, m->xfill, n_tok, DevRange{nullptr, m->ctr + CTR_EXITED, 0}, m->exit_tok, m->tok_seq,
                          m->tok_pos);
-      launch_standardize(st, m->dt, Xi, D, nullptr, act, mr, D, amode, eps, m->xn, D);
-      m->launches += 1;
       gemm(m, st, pr, 2, mrs, m->gemm_cls);
     } else {
       bool done = false;
@@ -1120,25 +1135,12 @@ static adept_status run_pass(adept_model* m, int n_tok, int batch, int prompt_le
         ex.par = pp; ex.layer = pl; ex.n_layers = N; ex.first = pl == 1; ex.test = pl >= 2;
         ex.metric = m->exit_metric; ex.norm_mode = amode; ex.eps = eps;
         done = streaming_gemm_exit(m, st, pr[0], mr, ex, m->gemm_cls) >= 0;
-        if (done) {
+        if (done)
           m->launches += 1;
-        } else {
-          // not taken: the exit step on its own first, then the product
-          xn_valid = launch_exit_small(st, pend.Xi, m->X_out, pend.Ii, pl == 1, D, m->ctr, pp, pend.rt,
-                                       m->row_tok[pp ^ 1], forced, pl, N, m->d_delta, pl >= 2, sim_out, m->exit_tok,
-                                       exit_w, m->X_in[pp ^ 1], m->I[pp ^ 1], m->hsm_s, m->hsm_prev, m->hsm_I, mr,
-                                       dgrows ? (bf16*)m->xn : nullptr, amode, eps, m->exit_metric, aao_len,
-                                       m->tok_pos, m->err_word) &&
-                     dgrows;
-          m->launches += 1;
-        }
-      }
-      if (!done) {
-        if (xn_valid)
-          gemm(m, st, pr, 1, mrs, m->gemm_cls);
         else
-          gemm_std(m, st, pr[0], mr, Xi, D, nullptr, amode, eps, m->gemm_cls);
+          exit_step(pl, pp, pend.Xi, pend.Ii, pend.rt);   // not taken: on its own first
       }
+      if (!done) gemm(m, st, pr, 1, mrs, m->gemm_cls);
     }
     // attention over every cached position of layer i
     {
@@ -1166,7 +1168,7 @@ static adept_status run_pass(adept_model* m, int n_tok, int batch, int prompt_le
     }
     gemm(m, st, &p, 1, &mr, m->gemm_cls);
     if (fam == ADEPT_FAMILY_BERT) {
-      launch_layernorm_inplace(st, m->X_out, act, mr, D, w.ln1_g, w.ln1_b, eps);
+      launch_layernorm_rows(st, m->dt, m->X_out, act, mr, D, w.ln1_g, w.ln1_b, eps, m->xn);   // and the FFN input
       m->launches += 1;
     }
     if (cross) {
@@ -1214,39 +1216,26 @@ static adept_status run_pass(adept_model* m, int n_tok, int batch, int prompt_le
       p.epi.act = fam == ADEPT_FAMILY_GPT2 ? ACT_GELU_TANH : ACT_GELU_ERF;
     }
     p.epi.bias = w.b_up; p.epi.out_t = m->hbuf; p.epi.ld_t = m->F;
-    gemm_std(m, st, p, mr, m->X_out, D, nullptr, amode, eps, m->gemm_cls, nullptr, ts_valid ? m->tile_stats : nullptr);
+    if (fam == ADEPT_FAMILY_BERT)
+      gemm(m, st, &p, 1, &mr, m->gemm_cls);
+    else
+      gemm_std(m, st, p, mr, m->X_out, D, nullptr, amode, eps, m->gemm_cls, nullptr, ts_valid ? m->tile_stats : nullptr);
     p.A = m->hbuf; p.lda = m->F; p.B = w.w_down; p.ldb = m->F; p.N = D; p.K = m->F;
     p.Bt = w.t_down; p.bt_nkb = cdiv(m->F, TW_KB);
     p.epi = epi_base(); p.epi.kind = EPI_RESID; p.epi.bias = w.b_down; p.epi.out_f32 = m->X_out; p.epi.ld_f32 = D;
     p.epi.resid = m->X_out; p.epi.ld_resid = D;
     gemm(m, st, &p, 1, &mr, m->gemm_cls);
     if (fam == ADEPT_FAMILY_BERT) {
-      launch_layernorm_inplace(st, m->X_out, act, mr, D, w.ln2_g, w.ln2_b, eps);
+      launch_layernorm_rows(st, m->dt, m->X_out, act, mr, D, w.ln2_g, w.ln2_b, eps, m->xn);
       m->launches += 1;
     }
     if (i < N) {
       // exit test (Sec. 4.1) for 2 <= i <= N-1, inertia update, compaction (App. I)
       const int test = i >= 2;
-      if (fuse_exit) {
+      if (fuse_exit)
         pend = {true, i, par, Xi, Ii, rt};
-        xn_valid = false;
-      } else if (n_tok <= EXIT_SMALL_MAX) {
-        xn_valid = launch_exit_small(st, Xi, m->X_out, Ii, i == 1, D, m->ctr, par, rt, m->row_tok[par ^ 1], forced, i,
-                                     N, m->d_delta, test, sim_out, m->exit_tok, exit_w, m->X_in[par ^ 1],
-                                     m->I[par ^ 1], m->hsm_s, m->hsm_prev, m->hsm_I, mr,
-                                     dgrows ? (bf16*)m->xn : nullptr, amode, eps, m->exit_metric, aao_len,
-                                     m->tok_pos, m->err_word) &&
-                   dgrows;
-        m->launches += 1;
-      } else {
-        launch_exit_decide(st, m->X_out, Ii, Xi, D, act, mr, rt, forced, i, N, m->d_delta, test, m->exit_metric,
-                           sim_out, m->flag, m->inv_norm, m->err_word);
-        launch_exit_scan(st, m->ctr, par, m->flag, rt, m->row_tok[par ^ 1], m->exit_tok, m->dst, exit_w, i, aao_len,
-                         m->tok_pos);
-        launch_exit_move(st, Xi, m->X_out, Ii, i == 1, D, m->ctr + CTR_ACTIVE + par, mr, m->dst, m->inv_norm,
-                         m->X_in[par ^ 1], m->I[par ^ 1], m->hsm_s, m->hsm_prev, m->hsm_I);
-        m->launches += 3;
-      }
+      else
+        exit_step(i, par, Xi, Ii, rt);
       if (!decode && test) {
         // HSM of the tokens that left at layer i (Sec. 4.2); their s~_N feeds the fills
         run_hsm(m, st, DevRange{m->ctr + CTR_PREFIX + i - 1, m->ctr + CTR_PREFIX + i, 0}, mr, n_tok);
