@@ -251,10 +251,12 @@ ADEPT_API adept_status adept_check_device_status(adept_model* m, void* stream);
  * (generation steps then run as direct launches).  GEMM_SIMT=1 routes GEMMs to the
  * SIMT kernels (cross-check).  DECODE_GRAPH (default 1): from its second call with a
  * given batch size, adept_decode_step replays a CUDA graph of the step captured once;
- * 0 launches every kernel directly.  DECODE_GEMM (default 1): single GEMMs of at most 16
- * rows (generation steps, output heads) of bf16 models run on the weight-streaming
- * generation-step kernel, with the input standardisation fused in; 0 routes them to the
- * tcgen05 kernel after a separate standardisation launch.  DECODE_STREAM (default 1): those
+ * 0 launches every kernel directly.  DECODE_GEMM (default 1): GEMMs of few rows of bf16 models
+ * (generation steps, short prompts, output heads, the mapper's products, small fills) run on the
+ * weight-streaming kernels: up to 8 rows on the generation-step kernels, with the input
+ * standardisation fused in (products of 128 MB of weights and more, and 9 to 128 rows: on the
+ * weight-streaming tcgen05 kernel, after a separate standardisation launch); 0 routes them to the
+ * tiled tcgen05 kernel.  DECODE_STREAM (default 1): those
  * weight-streaming GEMMs that are wide (at least 8192 outputs, or a grouped fill) and large
  * enough to stream (at least 8 MB of weights), and whose rows fit in shared memory, run on the
  * stream-K kernel (equal shares of the weight stream per SM, split tiles finished by the last

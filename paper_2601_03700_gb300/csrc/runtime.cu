@@ -7,6 +7,7 @@
 #include "gemm_tc.h"
 #include "gemm_decode.h"
 #include "gemm_stream.h"
+#include "gemm_swap.h"
 #include "model_view.h"
 #include "hsm_train.h"
 
@@ -348,10 +349,32 @@ static bool ensure_scratch(adept_model* m, size_t elems) {
 // tcgen05 path, but 16 tokens at 0.36 against 0.54, each CTA then staging a 64 KB operand slice).
 constexpr int DG_FILL_MAX_ROWS = 8;
 
+// Problems of 9 to 64 rows, and of up to 128 where a problem has at least 4 MB of weights, take the weight-streaming
+// tcgen05 kernel (GPT-2-small prompts of 128 tokens: 1334 us with that line, 1362 without it, 1459 at 8 MB and 1706
+// with none of them there; of 9 to 16 tokens the mma.sync kernels are slower at any size: 1192 us at 16, 971 here).
+// At up to 8 rows it takes single products of 128 MB and more (the SwiGLU input of a Llama-2-7B layer 30.8 -> 26.9 us
+// with its standardisation launch, FC2 / FC3 / head 64 -> 43); smaller ones gain nothing over the stream-K and cluster
+// kernels (a GPT-2-small step of 8 sequences: 543 against 510 us).
+constexpr long long SW_MIN_BYTES_MANY = 4ll << 20, SW_MIN_BYTES_FEW = 128ll << 20;
+// (Training products stay where they were: a step of few rows is bound by the optimiser, 1606 us on either path.)
+static bool sw_takes(const adept_model* m, int cls, int n_probs, const GemmProblem* p, const int* max_rows) {
+  if (cls == ADEPT_PROF_GEMM_TRAIN || m->dt != ADEPT_DTYPE_BF16 || m->force_simt || !m->use_dg || !tc_gemm_supported()) return false;
+  int rows = 0;
+  long long bytes = 0;
+  for (int i = 0; i < n_probs; ++i) {
+    if (!swap_gemm_supported(p[i], max_rows[i])) return false;
+    rows = std::max(rows, max_rows[i]);
+    bytes = std::max(bytes, (long long)p[i].N * p[i].K * 2);
+  }
+  if (rows > 8) return rows <= 64 || bytes >= SW_MIN_BYTES_MANY;
+  return n_probs == 1 && bytes >= SW_MIN_BYTES_FEW;
+}
+
 // The generation-step GEMM (gemm_decode.cu) takes single problems of at most DG_MAX_M rows.
-static bool dg_takes(const adept_model* m, int n_probs, const GemmProblem& p, int max_rows, const DgNorm* norm) {
+static bool dg_takes(const adept_model* m, int cls, int n_probs, const GemmProblem& p, int max_rows,
+                     const DgNorm* norm) {
   return m->dt == ADEPT_DTYPE_BF16 && !m->force_simt && m->use_dg && n_probs == 1 &&
-         decode_gemm_supported(p, max_rows, norm);
+         !sw_takes(m, cls, 1, &p, &max_rows) && decode_gemm_supported(p, max_rows, norm);
 }
 
 static DsWork ds_work(const adept_model* m) {
@@ -438,10 +461,18 @@ static void gemm(adept_model* m, cudaStream_t st, const GemmProblem* probs, int 
                  int cls, double flops = 0, double bytes = 0) {
   cudaEvent_t b = nullptr;
   prof_begin(m, cls, st, &b);
-  if (dg_takes(m, n_probs, probs[0], max_rows[0], nullptr) && streaming_gemm(m, st, probs[0], max_rows[0], nullptr, cls) >= 0) {
+  if (dg_takes(m, cls, n_probs, probs[0], max_rows[0], nullptr) && streaming_gemm(m, st, probs[0], max_rows[0], nullptr, cls) >= 0) {
     m->launches += 1;
     prof_end(m, cls, st, b, flops, bytes);
     return;
+  }
+  if (sw_takes(m, cls, n_probs, probs, max_rows)) {
+    SpanGuard sg(m, cls);
+    if (swap_gemm(st, probs, n_probs, max_rows, m->err_word) >= 0) {
+      m->launches += 1;
+      prof_end(m, cls, st, b, flops, bytes);
+      return;
+    }
   }
   if (m->dt == ADEPT_DTYPE_BF16 && !m->force_simt && tc_gemm_supported()) {
     const int nl = tc_gemm_grouped(st, probs, n_probs, max_rows, m->err_word);
@@ -476,7 +507,7 @@ static void gemm_std(adept_model* m, cudaStream_t st, const GemmProblem& p, int 
                      const int* in_rows, int mode, float eps, int cls, const float2* row_stats = nullptr,
                      const float2* tile_stats = nullptr) {
   const DgNorm nrm{X, ldx, in_rows, mode, eps, row_stats, tile_stats};
-  if (dg_takes(m, 1, p, max_rows, &nrm)) {
+  if (dg_takes(m, cls, 1, p, max_rows, &nrm)) {
     cudaEvent_t b = nullptr;
     prof_begin(m, cls, st, &b);
     if (streaming_gemm(m, st, p, max_rows, &nrm, cls) >= 0) {
@@ -1163,7 +1194,7 @@ static adept_status run_pass(adept_model* m, int n_tok, int batch, int prompt_le
     bool ts_valid = false;   // the O projection leaves the tile statistics of X_out for the FFN input
     if (dgrows) {
       p.epi.tile_stats = m->tile_stats;
-      ts_valid = dg_takes(m, 1, p, mr, nullptr);
+      ts_valid = dg_takes(m, m->gemm_cls, 1, p, mr, nullptr);
       if (!ts_valid) p.epi.tile_stats = nullptr;
     }
     gemm(m, st, &p, 1, &mr, m->gemm_cls);
@@ -1200,7 +1231,7 @@ static adept_status run_pass(adept_model* m, int n_tok, int batch, int prompt_le
       ts_valid = false;   // the statistics of the FFN input now come from this product
       if (dgrows) {
         pc.epi.tile_stats = m->tile_stats;
-        ts_valid = dg_takes(m, 1, pc, mr, nullptr);
+        ts_valid = dg_takes(m, m->gemm_cls, 1, pc, mr, nullptr);
         if (!ts_valid) pc.epi.tile_stats = nullptr;
       }
       gemm(m, st, &pc, 1, &mr, m->gemm_cls);
@@ -1268,7 +1299,8 @@ static adept_status run_pass(adept_model* m, int n_tok, int batch, int prompt_le
     // one weight-streaming launch over the skipped layers when the rows fit it, else the
     // grouped tcgen05 GEMM
     bool done = false;
-    if (m->dt == ADEPT_DTYPE_BF16 && m->use_dg && !m->force_simt && n_tok <= DG_MAX_M) {
+    if (m->dt == ADEPT_DTYPE_BF16 && m->use_dg && !m->force_simt && n_tok <= DG_MAX_M &&
+        !sw_takes(m, ADEPT_PROF_KV_FILL, (int)probs.size(), probs.data(), mrs.data())) {
       cudaEvent_t b = nullptr;
       prof_begin(m, ADEPT_PROF_KV_FILL, st, &b);
       done = streaming_gemm_grouped(m, st, probs.data(), (int)probs.size(), n_tok) >= 0;
@@ -1959,7 +1991,8 @@ adept_status adept_skip_kv_fill(adept_model* m, int n_tokens, const void* d_h_ma
   // algorithmic work of this launch is only known on the device; the benchmark supplies it.
   // A few tokens: one weight-streaming launch over the layers; else the grouped tcgen05 GEMM.
   bool done = false;
-  if (m->dt == ADEPT_DTYPE_BF16 && m->use_dg && !m->force_simt && n_tokens <= DG_MAX_M) {
+  if (m->dt == ADEPT_DTYPE_BF16 && m->use_dg && !m->force_simt && n_tokens <= DG_MAX_M &&
+      !sw_takes(m, ADEPT_PROF_KV_FILL, (int)probs.size(), probs.data(), mrs.data())) {
     cudaEvent_t b = nullptr;
     prof_begin(m, ADEPT_PROF_KV_FILL, st, &b);
     done = streaming_gemm_grouped(m, st, probs.data(), (int)probs.size(), n_tokens) >= 0;
@@ -2021,7 +2054,7 @@ adept_status adept_check_device_status(adept_model* m, void* stream) {
 adept_status adept_set_wait_limit(int64_t cycles) {
   if (cycles < 0) return fail(nullptr, ADEPT_ERR_INVALID_ARG, "wait limit %lld < 0", (long long)cycles);
   const long long v = cycles == 0 ? WAIT_LIMIT_DEFAULT : (long long)cycles;
-  for (cudaError_t e : {set_wait_limit_tc(v), set_wait_limit_dg(v), set_wait_limit_ds(v)})
+  for (cudaError_t e : {set_wait_limit_tc(v), set_wait_limit_dg(v), set_wait_limit_ds(v), set_wait_limit_sw(v)})
     if (e != cudaSuccess) return fail(nullptr, ADEPT_ERR_CUDA, "setting the wait limit: %s", cudaGetErrorString(e));
   return ADEPT_OK;
 }
