@@ -1,6 +1,7 @@
-// SIMT GEMM (fp32 FMA) with a separate epilogue pass.  This is the path of the fp32
-// models and the cross-check of the tensor-core GEMM; its epilogue semantics are the
-// reference for the fused tcgen05 epilogue.
+// fp32-FMA GEMMs: the path of the fp32 models, and the cross-check of the tensor-core GEMM.
+// f32_rows_kernel (fp32, the epilogue fused) takes passes of up to F32_ROWS_MAX rows;
+// gemm_simt_kernel, a 64 x 64 tile with a separate epilogue pass, the rest and bf16 operands (its
+// epilogue semantics are the reference for the fused tcgen05 epilogue).
 #define ADEPT_TU_ID 2
 #include "common.cuh"
 #include "kernels.h"
@@ -71,6 +72,173 @@ __global__ void epilogue_kernel(Epi e, const float* __restrict__ C, int ldc, Dev
     for (int j = 0; j < 32; ++j) v[j] = (c0 + j < N) ? c[c0 + j] : 0.f;
     epi_chunk32<T>(e, ra, c0, N, v, rr);
   }
+}
+
+// C[r, n] = sum_k A[r, k] * B[n, k] for a few rows, fp32, with the fused epilogue.
+//
+// The fp32 models are small: a product's weights lie in L2 and its time is latency. The 64 x 64 tile
+// left most SMs idle (4 CTAs for 64 rows x 256 outputs) and walked K in 16-element steps with two
+// barriers each, and its epilogue was a launch of its own. Here a warp takes 4 features x 8 rows with
+// its lanes split over K: every weight of a 512-element slice of K is read once into registers, as
+// float4 and before the programmatic-dependent-launch wait (`ahead`: the operand is a weight that no
+// preceding kernel writes), so that after the wait only the rows are to come. WK warps of the CTA
+// share a long K; the 32 sums of a warp meet by a transposing butterfly (31 shuffles, lane = sum).
+// The tile of 4 * 8 / WK features x 8 rows goes through the epilogue one element per thread.
+// Measured (tiny configuration: D = 256, FFN 1024, mapper 1024 / 2048; kernel times without launch overlap): one row
+// 43 us a product on average plus 4 for its epilogue launch -> 2.3 to 5.0; its 64-token prompt and 16 steps 20.4 ->
+// 2.0 ms.
+constexpr int FR_THREADS = 256, FR_R = 8, FR_F = 4, FR_KC = 512;
+// The bound: prompt passes of a model of D = 1024 (4 layers, mapper 4096 / 8192), all rows to full depth, take
+// 1.15 / 2.24 / 4.43 / 9.20 ms at 64 / 128 / 256 / 512 rows here and 4.59 / 4.68 / 5.85 / 8.53 on the tile.
+constexpr int F32_ROWS_MAX = 256;
+
+template <int WK, int KIND>
+__global__ void __launch_bounds__(FR_THREADS) f32_rows_kernel(const float* __restrict__ A, int lda,
+                                                              const float* __restrict__ B, int ldb, DevRange rows,
+                                                              int N, int K, Epi e, int ahead) {
+  KT_BEGIN();
+  constexpr int WF = FR_THREADS / 32 / WK, FT = FR_F * WF;   // feature groups, features of the CTA
+  constexpr int NJ = FR_KC / 128;                            // float4 per lane of a slice
+  __shared__ float s_part[WK][FR_R][FT + 1];
+  __shared__ float s_v[FR_R][FT + 1];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, wf = warp % WF, wk = warp / WF;
+  // feature of the CTA's local index: consecutive, or (SwiGLU: gate and up rows interleaved in blocks
+  // of 16) half of them gates and half the matching ups
+  auto feature = [&](int lf) {
+    if (KIND != EPI_SWIGLU || FT == 32) return (int)blockIdx.x * FT + lf;
+    constexpr int PARTS = 32 / FT, H = FT / 2;
+    const int block = blockIdx.x / PARTS, part = blockIdx.x % PARTS;
+    return block * 32 + part * H + (lf < H ? lf : 16 + lf - H);
+  };
+  float4 w[FR_F][NJ];
+  auto load_w = [&](int k0) {
+#pragma unroll
+    for (int f = 0; f < FR_F; ++f) {
+      const int n = feature(wf * FR_F + f);
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) {
+        const int k = k0 + (j * 32 + lane) * 4;
+        w[f][j] = n < N && k < K ? *reinterpret_cast<const float4*>(B + (size_t)n * ldb + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    }
+  };
+  if (ahead) load_w(wk * FR_KC);
+  pdl_wait();
+  KT_WAITED();
+  pdl_launch_dependents();
+  const int rb = rows.b(), M = rows.e() - rb, r0 = blockIdx.y * FR_R;
+  if (r0 >= M) return;
+  const int nr = min(FR_R, M - r0);
+  float acc[FR_F * FR_R];
+#pragma unroll
+  for (int i = 0; i < FR_F * FR_R; ++i) acc[i] = 0.f;
+  for (int k0 = wk * FR_KC; k0 < K; k0 += WK * FR_KC) {
+    if (!ahead || k0 >= WK * FR_KC) load_w(k0);
+#pragma unroll
+    for (int r = 0; r < FR_R; ++r) {
+      if (r >= nr) break;
+      const float* a = A + (size_t)(rb + r0 + r) * lda;
+      float4 x[NJ];
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) {
+        const int k = k0 + (j * 32 + lane) * 4;
+        x[j] = k < K ? *reinterpret_cast<const float4*>(a + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+#pragma unroll
+      for (int f = 0; f < FR_F; ++f)
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) {
+          float& c = acc[f * FR_R + r];
+          c = fmaf(x[j].x, w[f][j].x, c);
+          c = fmaf(x[j].y, w[f][j].y, c);
+          c = fmaf(x[j].z, w[f][j].z, c);
+          c = fmaf(x[j].w, w[f][j].w, c);
+        }
+    }
+  }
+  // lane i ends with sum i = (feature i >> 3, row i & 7)
+#pragma unroll
+  for (int o = 16; o; o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < o; ++i) {
+      const float give = up ? acc[i] : acc[i + o], keep = up ? acc[i + o] : acc[i];
+      acc[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+  }
+  s_part[wk][lane & (FR_R - 1)][wf * FR_F + (lane >> 3)] = acc[0];
+  __syncthreads();
+  const int r = threadIdx.x / FT, lf = threadIdx.x % FT, ra = rb + r0 + r, c = feature(lf);
+  const bool mine = r < nr && c < N;
+  float v = 0.f;
+  if (mine) {
+#pragma unroll
+    for (int k = 0; k < WK; ++k) v += s_part[k][r][lf];
+    if (e.bias) v += e.bias[c];
+  }
+  if (KIND == EPI_SWIGLU || KIND == EPI_QKV) {   // the other member of a pair
+    if (r < FR_R) s_v[r][lf] = v;
+    __syncthreads();
+  }
+  if (!mine) return;
+  if (KIND == EPI_F32) {
+    e.out_f32[(size_t)ra * e.ld_f32 + c] = v;
+  } else if (KIND == EPI_ACT) {
+    v = apply_act(e.act, v);
+    ((float*)e.out_t)[(size_t)ra * e.ld_t + c] = v;
+    if (e.out_f32) e.out_f32[(size_t)ra * e.ld_f32 + c] = v;
+  } else if (KIND == EPI_RESID) {
+    e.out_f32[(size_t)ra * e.ld_f32 + c] = e.resid[(size_t)ra * e.ld_resid + c] + v;
+  } else if (KIND == EPI_SWIGLU) {
+    if ((c & 31) < 16)
+      ((float*)e.out_t)[(size_t)ra * e.ld_t + (c >> 5) * 16 + (c & 15)] = silu_f(v) * s_v[r][lf + FT / 2];
+  } else {   // EPI_QKV / EPI_KV: q -> out_t, k / v -> the row's cache slot; rotary pairs in adjacent features
+    const EpiRow rr = epi_row(e, ra);
+    const int dh = e.head_dim, half = dh >> 1, nq = e.n_q_cols, nkv = e.n_kv_cols;
+    const int base = c < nq ? 0 : c < nq + nkv ? nq : nq + nkv, h = (c - base) / dh, d = (c - base) - h * dh;
+    int od = d;
+    if (e.rope && base < nq + nkv) {
+      const int ip = d >> 1;
+      const float2 cs = e.rope_table[(size_t)rr.pos * half + ip];
+      const float o = s_v[r][lf ^ 1];
+      // (x1, x2) -> (x1 cos - x2 sin, x2 cos + x1 sin)
+      v = (d & 1) ? v * cs.x + o * cs.y : v * cs.x - o * cs.y;
+      od = (d & 1) ? ip + half : ip;
+    }
+    if (c < nq)
+      ((float*)e.out_t)[(size_t)ra * e.ld_t + h * dh + od] = v;
+    else if (rr.cbase >= 0)
+      ((float*)(c < nq + nkv ? e.cache.k : e.cache.v))[rr.cbase + (size_t)h * e.cache.head_stride() + od] = v;
+  }
+}
+
+template <int WK>
+static void f32_rows_go(cudaStream_t st, const GemmProblem& p, int max_rows, bool ahead) {
+  constexpr int FT = FR_F * (FR_THREADS / 32 / WK);
+  const dim3 grid(cdiv(p.N, FT), cdiv(max_rows, FR_R));
+#define GO(KIND)                                                                                                  \
+  launch_k(f32_rows_kernel<WK, KIND>, grid, FR_THREADS, 0, st, (const float*)p.A, p.lda, (const float*)p.B, p.ldb, \
+           p.rows, p.N, p.K, p.epi, ahead ? 1 : 0)
+  switch (p.epi.kind) {
+    case EPI_F32: GO(EPI_F32); break;
+    case EPI_ACT: GO(EPI_ACT); break;
+    case EPI_RESID: GO(EPI_RESID); break;
+    case EPI_SWIGLU: GO(EPI_SWIGLU); break;
+    default: GO(EPI_QKV); break;   // EPI_KV: no query columns
+  }
+#undef GO
+}
+
+bool gemm_f32_rows(cudaStream_t st, const GemmProblem& p, int max_rows, bool ahead) {
+  if (max_rows < 1 || max_rows > F32_ROWS_MAX || p.N < 1 || p.K < 1) return false;
+  if ((p.K | p.lda | p.ldb) % 4 || (((uintptr_t)p.A | (uintptr_t)p.B) & 15)) return false;
+  if (p.epi.kind < EPI_F32 || p.epi.kind > EPI_KV) return false;
+  if ((p.epi.kind == EPI_SWIGLU || p.epi.kind >= EPI_QKV) && p.N % 32) return false;
+  // K slices of 512 over 1, 2 or 4 warps
+  if (p.K <= FR_KC) f32_rows_go<1>(st, p, max_rows, ahead);
+  else if (p.K <= 2 * FR_KC) f32_rows_go<2>(st, p, max_rows, ahead);
+  else f32_rows_go<4>(st, p, max_rows, ahead);
+  return true;
 }
 
 void launch_gemm_simt(cudaStream_t st, int dt, const GemmProblem& p, int max_rows, float* scratch) {

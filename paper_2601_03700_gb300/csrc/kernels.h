@@ -106,6 +106,9 @@ void launch_read_kv(cudaStream_t st, int dt, KVCacheView c, int layer0, int seq,
 
 // GEMMs.  SIMT path: C = A B^T into fp32 scratch, then the epilogue kernel.
 void launch_gemm_simt(cudaStream_t st, int dt, const GemmProblem& p, int max_rows, float* scratch);
+// fp32 problem of few rows in one launch (no scratch); ahead: B is a weight that no kernel still
+// running may write, read before the dependency wait.  False when the shape is not taken.
+bool gemm_f32_rows(cudaStream_t st, const GemmProblem& p, int max_rows, bool ahead);
 // Attention of the active query rows over the paged cache of one layer.
 // decode_keys > 0 (generation step, one query row per sequence): split-KV kernel over at
 // most decode_keys keys, using ws (>= rows * heads * ATTN_MAX_SPLIT * (head_dim + 2) floats)
