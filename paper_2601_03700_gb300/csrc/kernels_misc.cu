@@ -1105,18 +1105,24 @@ __global__ void to_f32_kernel(const T* src, float* dst, int n) {
   if (i < n) dst[i] = to_f(src[i]);
 }
 
-// Copy n_pos positions of one sequence / layer out of the paged cache.
-template <typename T>
-__global__ void read_kv_kernel(KVCacheView c, int layer0, int seq, int pos0, int n_pos, T* ko, T* vo) {
+// Copy n_pos positions of one sequence / layer out of the paged cache: a copy bound by HBM / L2.  A
+// thread takes one piece (P: 16 bytes, or one element where the caller's buffers allow no more) of K and
+// of V, so that a warp moves whole (position, head) rows and both its loads are under way together.
+// 2000 positions of 32 x 128 (33 MB out): 37 us on one element a thread and turn (with the block table
+// read for each), 12.8 here; the bytes take 9.6 at the measured HBM rate.
+template <typename P>
+__global__ void __launch_bounds__(256) read_kv_kernel(KVCacheView c, int row_bytes, int layer0, int seq, int pos0,
+                                                      int n_pos, P* __restrict__ ko, P* __restrict__ vo) {
   PDL_ENTRY();
-  const int p = blockIdx.x;
-  if (p >= n_pos) return;
-  const int per = c.n_kv_heads * c.head_dim;
-  for (int e = threadIdx.x; e < per; e += blockDim.x) {
-    const int h = e / c.head_dim, d = e % c.head_dim;
-    const size_t off = c.offset(layer0, seq, pos0 + p, h) + d;
-    ko[(size_t)p * per + e] = ((const T*)c.k)[off];
-    vo[(size_t)p * per + e] = ((const T*)c.v)[off];
+  const int per_head = row_bytes / (int)sizeof(P);          // pieces of a (position, head) row
+  const int per_pos = per_head * c.n_kv_heads;
+  const long long total = (long long)per_pos * n_pos, step = (long long)gridDim.x * blockDim.x;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += step) {
+    const int p = (int)(i / per_pos), e = (int)(i - (long long)p * per_pos), h = e / per_head;
+    const size_t off = c.offset(layer0, seq, pos0 + p, h) / c.head_dim * per_head + (e - h * per_head);
+    const P k = reinterpret_cast<const P*>(c.k)[off], v = reinterpret_cast<const P*>(c.v)[off];
+    ko[i] = k;
+    vo[i] = v;
   }
 }
 
@@ -1396,8 +1402,13 @@ void launch_to_f32(cudaStream_t st, int dt, const void* src, float* dst, int n) 
 void launch_read_kv(cudaStream_t st, int dt, KVCacheView c, int layer0, int seq, int pos0, int n_pos, void* ko,
                     void* vo) {
   if (n_pos <= 0) return;
-  if (dt == 1) launch_k(read_kv_kernel<bf16>, n_pos, 256, 0, st, c, layer0, seq, pos0, n_pos, (bf16*)ko, (bf16*)vo);
-  else launch_k(read_kv_kernel<float>, n_pos, 256, 0, st, c, layer0, seq, pos0, n_pos, (float*)ko, (float*)vo);
+  const int esz = dt == 1 ? 2 : 4, row_bytes = c.head_dim * esz;   // head_dim 32, 64 or 128: whole 16-byte pieces
+  const bool wide = (((uintptr_t)ko | (uintptr_t)vo) & 15) == 0;
+  const long long pieces = (long long)n_pos * c.n_kv_heads * (row_bytes / (wide ? 16 : esz));
+  const int grid = (int)std::min<long long>((pieces + 255) / 256, 1 << 20);
+  if (wide) launch_k(read_kv_kernel<uint4>, grid, 256, 0, st, c, row_bytes, layer0, seq, pos0, n_pos, (uint4*)ko, (uint4*)vo);
+  else if (dt == 1) launch_k(read_kv_kernel<bf16>, grid, 256, 0, st, c, row_bytes, layer0, seq, pos0, n_pos, (bf16*)ko, (bf16*)vo);
+  else launch_k(read_kv_kernel<float>, grid, 256, 0, st, c, row_bytes, layer0, seq, pos0, n_pos, (float*)ko, (float*)vo);
 }
 
 // Tile-contiguous weight copy: one thread per 16-byte piece of the destination.  Piece q of
