@@ -1028,41 +1028,25 @@ __global__ void __launch_bounds__(512) fill_plan_kernel(const T* h, int D, const
     plan_row(h + (size_t)row * D, xs + (size_t)s_slot[row] * D, D, mode, eps, lane);
 }
 
+// Larger calls: a warp per row takes the row's place in its exit layer's bucket and standardises it
+// (the row in registers). 2000 rows of 4096: 23.9 us with a CTA per row that read it again, an element
+// a thread, for each reduction; 9.0 here (5 at the measured HBM rate).
 template <typename T>
-__global__ void fill_scatter_kernel(const T* h, int n, int D, const int* exit_layer, int n_layers, const int* start,
-                                    int* cursor, int* sorted_tok, T* xs, int mode, float eps) {
+__global__ void __launch_bounds__(128) fill_scatter_kernel(const T* h, int n, int D, const int* exit_layer,
+                                                           int n_layers, const int* start, int* cursor,
+                                                           int* sorted_tok, T* xs, int mode, float eps) {
   PDL_ENTRY();
-  __shared__ float red[32];
-  __shared__ int s_slot;
-  const int j = blockIdx.x;
+  const int j = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (j >= n) return;
-  if (threadIdx.x == 0) {
+  int slot = 0;
+  if (lane == 0) {
     int l = exit_layer[j];
     if (l < 1 || l > n_layers) l = n_layers;
-    s_slot = start[l] + atomicAdd(&cursor[l], 1);
-    sorted_tok[s_slot] = j;
+    slot = start[l] + atomicAdd(&cursor[l], 1);
+    sorted_tok[slot] = j;
   }
-  __syncthreads();
-  const int slot = s_slot;
-  const T* x = h + (size_t)j * D;
-  T* o = xs + (size_t)slot * D;
-  if (mode == NORM_COPY) {
-    for (int d = threadIdx.x; d < D; d += blockDim.x) o[d] = x[d];
-    return;
-  }
-  float mu = 0.f;
-  if (mode == NORM_LN) {
-    float s = 0.f;
-    for (int d = threadIdx.x; d < D; d += blockDim.x) s += to_f(x[d]);
-    mu = block_sum(s, red) / D;
-  }
-  float s2 = 0.f;
-  for (int d = threadIdx.x; d < D; d += blockDim.x) {
-    const float c = to_f(x[d]) - mu;
-    s2 += c * c;
-  }
-  const float rstd = rsqrtf(block_sum(s2, red) / D + eps);
-  for (int d = threadIdx.x; d < D; d += blockDim.x) o[d] = from_f<T>((to_f(x[d]) - mu) * rstd);
+  slot = __shfl_sync(0xffffffffu, slot, 0);
+  plan_row(h + (size_t)j * D, xs + (size_t)slot * D, D, mode, eps, lane);
 }
 
 // ---------------------------------------------------------------------------
@@ -1375,10 +1359,10 @@ int launch_fill_sort(cudaStream_t st, int dt, const void* h, int n, int D, const
              cursor, sorted_tok, (float*)xs, mode, eps, err);
   if (n <= FILL_PLAN_ROWS) return 1;   // placed and standardised by the plan kernel
   if (dt == 1)
-    launch_k(fill_scatter_kernel<bf16>, n, 256, 0, st, (const bf16*)h, n, D, exit_layer, n_layers, start, cursor,
+    launch_k(fill_scatter_kernel<bf16>, cdiv(n, 4), 128, 0, st, (const bf16*)h, n, D, exit_layer, n_layers, start, cursor,
                                                  sorted_tok, (bf16*)xs, mode, eps);
   else
-    launch_k(fill_scatter_kernel<float>, n, 256, 0, st, (const float*)h, n, D, exit_layer, n_layers, start, cursor,
+    launch_k(fill_scatter_kernel<float>, cdiv(n, 4), 128, 0, st, (const float*)h, n, D, exit_layer, n_layers, start, cursor,
                                                   sorted_tok, (float*)xs, mode, eps);
   return 2;
 }
