@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
     uint8_t* dst0 = kw ? sK : sV;
     int issued = 0;
     bool ok = true;
-    if (kw && lane == 0) {
+    if (kw && elect_one()) {
       mbar_expect_tx(&q_full, (uint32_t)L::Q_BYTES);
       for (int hf = 0; hf < L::HALVES; ++hf) tma_load_2d(&p.qmap, &q_full, sQ + hf * AT_BM * 128, h * DH + hf * 64, r0);
     }
@@ -312,7 +312,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
         for (int b = 0; b < AT_BN / 16; ++b) rows8[b] = __shfl_sync(0xffffffffu, myrow, b);
         if (it >= 2 && !(ok = at_wait_warp(&empty[s], (uint32_t)(((it >> 1) - 1) & 1), abort_flag, p.err, wlim)))
           break;
-        if (lane == 0) {
+        if (elect_one()) {
           mbar_expect_tx(&full[s], (uint32_t)L::KV_BYTES);
           for (int b = 0; b < AT_BN / 16; ++b)
             for (int hf = 0; hf < L::HALVES; ++hf)
@@ -347,7 +347,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
     auto issue_s = [&](int it) {
       const int s = it & 1;
       tc_fence_after();
-      if (lane == 0) {
+      if (elect_one()) {
         const uint32_t d = tmem + (uint32_t)(s * 128);
 #pragma unroll
         for (int kk = 0; kk < DH / 16; ++kk) {
@@ -398,7 +398,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
             __syncwarp();
           }
           tc_fence_after();
-          if (lane == 0) {
+          if (elect_one()) {
             const uint32_t pa = tmem + 384 + (uint32_t)((npv & 1) * 64);   // P of this tile in TMEM
 #pragma unroll
             for (int kk = 0; kk < AT_BN / 16; ++kk) {
@@ -433,7 +433,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
       ok = __all_sync(0xffffffffu, ok) != 0;
     }
     // every MMA issued has completed before tensor memory is freed
-    if (lane == 0) {
+    if (elect_one()) {
       umma_commit(&drain);
       const long long t0 = clock64();
       while (!mbar_try_wait(&drain, 0) && clock64() - t0 < AT_DRAIN_CYCLES) {

@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(SW_THREADS) gemm_swap_kernel(const __grid_cons
     }
   } else {
     if (warp == 0) {
-      if (lane == 0) {
+      if (elect_one()) {
         // ------------------------------------------------------------ TMA producer
         int s = 0, n = 0;   // slot and its use number
         uint32_t issued = 0, last_par = 0;
@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(SW_THREADS) gemm_swap_kernel(const __grid_cons
           if (issued >> k & 1u) land(k, (last_par >> k) & 1u);
       }
     } else if (warp == 1) {
-      if (lane == 0) {
+      if (elect_one()) {
         // ------------------------------------------------------------ MMA issuer
         // kind::f16: D fp32, A and B bf16, both K-major, M = 128, N = the live rows
         const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(((M + 15) >> 4) * 2) << 17) |
