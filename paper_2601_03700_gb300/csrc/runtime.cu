@@ -7,6 +7,7 @@
 #include "gemm_tc.h"
 #include "gemm_decode.h"
 #include "gemm_stream.h"
+#include "gemm_pair.h"
 #include "gemm_swap.h"
 #include "model_view.h"
 #include "hsm_train.h"
@@ -475,7 +476,8 @@ static void gemm(adept_model* m, cudaStream_t st, const GemmProblem* probs, int 
     }
   }
   if (m->dt == ADEPT_DTYPE_BF16 && !m->force_simt && tc_gemm_supported()) {
-    const int nl = tc_gemm_grouped(st, probs, n_probs, max_rows, m->err_word);
+    int nl = pair_gemm(st, probs, n_probs, max_rows, m->err_word);
+    if (nl < 0) nl = tc_gemm_grouped(st, probs, n_probs, max_rows, m->err_word);
     if (nl >= 0) {
       m->launches += nl;
       prof_end(m, cls, st, b, flops, bytes);
@@ -2059,7 +2061,8 @@ adept_status adept_check_device_status(adept_model* m, void* stream) {
 adept_status adept_set_wait_limit(int64_t cycles) {
   if (cycles < 0) return fail(nullptr, ADEPT_ERR_INVALID_ARG, "wait limit %lld < 0", (long long)cycles);
   const long long v = cycles == 0 ? WAIT_LIMIT_DEFAULT : (long long)cycles;
-  for (cudaError_t e : {set_wait_limit_tc(v), set_wait_limit_dg(v), set_wait_limit_ds(v), set_wait_limit_sw(v)})
+  for (cudaError_t e : {set_wait_limit_tc(v), set_wait_limit_dg(v), set_wait_limit_ds(v), set_wait_limit_sw(v),
+                        set_wait_limit_pg(v)})
     if (e != cudaSuccess) return fail(nullptr, ADEPT_ERR_CUDA, "setting the wait limit: %s", cudaGetErrorString(e));
   return ADEPT_OK;
 }

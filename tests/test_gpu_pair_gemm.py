@@ -1,0 +1,60 @@
+"""The paired tcgen05 GEMM (more than 128 token rows) against the oracle: row counts at the edges of its 256-row tiles and
+of its CTAs' 128-row halves, inner sizes that are no multiple of its 64-wide k-blocks or of whole tiles, live row counts from
+none to all (which move its tile width), grouped fills of many layers, and the logits of a ragged vocabulary."""
+import numpy as np
+import pytest
+import torch
+
+import synth
+from oracle import adept_oracle as O
+from parity_utils import Pair, assert_rows_close, compare_prefill
+
+import paper_2601_03700_gb300 as adept
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    adept.load_library()
+
+
+def config(family, B, P, **kw):
+    base = dict(family=family, n_layers=5, d_model=320, n_heads=5, head_dim=64, d_ffn=464, vocab=1003, max_pos=320,
+                n_classes=3 if family == synth.BERT else 0, dtype="bf16", hsm_m1=584, hsm_m2=1096, max_batch=B,
+                max_seq=max(P + 4, 16), max_pass_tokens=max(B * P, B), block_shuffle_seed=5)
+    base.update(kw)
+    return synth.ModelConfig(**base)
+
+
+@pytest.mark.parametrize("family", [synth.LLAMA, synth.GPT2, synth.BERT])
+@pytest.mark.parametrize("B,P", [(1, 129), (5, 51), (1, 257), (3, 128), (131, 4)])
+def test_pair_gemm_prompt_matches_oracle(family, B, P):
+    pair = Pair(config(family, B, P), seed=110 + P)
+    tokens = synth.make_tokens(111, B, P, 1003).numpy()
+    forced = synth.forced_exits_uniform(112 + P, B * P, 2, 5).numpy().reshape(B, P)
+    compare_prefill(pair, tokens, 0.9, forced)
+    compare_prefill(pair, tokens, -2.0)      # every token leaves at layer 2: no rows after it
+    pair.close()
+
+
+@pytest.mark.parametrize("n", [129, 300])
+def test_pair_gemm_grouped_fill_matches_oracle(n):
+    cfg = config(synth.LLAMA, 1, 300, n_layers=9)
+    pair = Pair(cfg, seed=117)
+    adept.adept_seq_reserve(pair.gm.h, [300])
+    h = synth.make_mapped_states(118, n, cfg.d_model)
+    el = synth.forced_exits_uniform(119, n, 1, 9).numpy()
+    pos = np.random.RandomState(3).permutation(300)[:n]
+    adept.adept_skip_kv_fill(pair.gm.h, n, h.cuda(), torch.as_tensor(el, dtype=torch.int32).cuda(),
+                             torch.zeros(n, dtype=torch.int32, device="cuda"),
+                             torch.as_tensor(pos, dtype=torch.int32).cuda())
+    pair.gm.check()
+    want = O.skip_kv_fill(pair.om, h.double().numpy(), el, pos)
+    for r, (k, v, sel) in want.items():
+        gk, gv = pair.gpu_kv(r, 0, 300)
+        assert_rows_close(gk[pos[sel]], k, pair.tol, f"K layer {r}")
+        assert_rows_close(gv[pos[sel]], v, pair.tol, f"V layer {r}")
+    pair.close()
