@@ -265,6 +265,27 @@ __device__ __forceinline__ float block_sum(float v, float* red) {
 }
 
 __device__ __forceinline__ float gelu_erf_f(float x) { return 0.5f * x * (1.f + erff(x * 0.70710678118654752f)); }
+// The same for results that are rounded to bf16: x Phi(x) = max(x, 0) - z Phi(-z), z = |x|, with
+// Phi(-z) = exp(-z^2 / 2) R(t), t = 1 / (1 + 0.33 z), and R a polynomial fitted to 0.5 erfcx(z / sqrt 2) over z in [0, 7]
+// (relative error 5e-8; least squares re-weighted towards equal extremes). Two hardware approximations (1 / d, 2^a) and 17
+// instructions where erff takes about 60. Against 64 bits: 3.4e-8 of the result's norm over N(0, 1) and 1.0e-7 over
+// N(0, 0.1), the erff form 3.8e-8 in both; the rounding to bf16 is 1.7e-3. Below -3 it keeps 6 digits, the erff form 1.
+// NaN and the infinities as the erff form gives them.
+__device__ __forceinline__ float gelu_erf_bf(float x) {
+  const float z = fminf(fabsf(x), 20.f), d = fmaf(0.33f, z, 1.f), a = z * (z * -0.72134752044448170f);
+  float t, e;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(d));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(a));
+  float r = 0.04947014978f;
+  r = fmaf(r, t, -0.23992625065f);
+  r = fmaf(r, t, 0.37131077812f);
+  r = fmaf(r, t, -0.13445004592f);
+  r = fmaf(r, t, 0.21082835485f);
+  r = fmaf(r, t, 0.10797602751f);
+  r = fmaf(r, t, 0.13499328363f);
+  r = fmaf(r, t, -0.00020231069264f);
+  return fmaf(0.5f, fabsf(x), 0.5f * x) - z * e * r;
+}
 __device__ __forceinline__ float gelu_tanh_f(float x) {
   return 0.5f * x * (1.f + tanhf(0.79788456080286536f * (x + 0.044715f * x * x * x)));
 }

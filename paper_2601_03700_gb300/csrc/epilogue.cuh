@@ -60,6 +60,11 @@ __device__ __forceinline__ EpiRow epi_row(const Epi& e, int ra) {
   return r;
 }
 
+// One pair turned by (cos, sin), its operations fixed so that every kernel rounds alike.
+__device__ __forceinline__ float2 rope_turn(float x1, float x2, float co, float si) {
+  return make_float2(fmaf(x1, co, -__fmul_rn(x2, si)), fmaf(x2, co, __fmul_rn(x1, si)));
+}
+
 // Rotary embedding of 16 adjacent pairs (columns 2j, 2j+1 -> features i0+j, i0+j+half),
 // written as two runs of 16 at dst[i0] and dst[i0 + half].
 template <typename T>
@@ -69,8 +74,9 @@ __device__ __forceinline__ void rope_pairs(T* dst, int i0, int half, const float
   for (int j = 0; j < 16; ++j) {
     const float2 cs = tab[i0 + j];
     const float x1 = v[2 * j], x2 = v[2 * j + 1];
-    a[j] = x1 * cs.x - x2 * cs.y;
-    b[j] = x2 * cs.x + x1 * cs.y;
+    const float2 y = rope_turn(x1, x2, cs.x, cs.y);
+    a[j] = y.x;
+    b[j] = y.y;
   }
   store16<T>(dst + i0, a);
   store16<T>(dst + i0 + half, b);

@@ -8,13 +8,16 @@
 //    active, or that leave, at a layer): the width whose whole waves of tiles take the least time. 2048 rows x 4096 outputs
 //    are 2 full waves of 224 columns; in tiles of 256 they are 1.7. One launch serves every count.
 //  * 8 epilogue warps per CTA (two per TMEM lane quarter, taking the tile's 32-column chunks in turn). A chunk leaves tensor
-//    memory a row per lane and is turned around in shared memory, so that residuals, biases and results move as whole
-//    128-byte (bf16: 64-byte) row pieces; a row per lane took a transaction per lane.
+//    memory a row per lane and is turned around in shared memory, so that residuals and results move as whole 128-byte (bf16:
+//    64-byte) row pieces; a row per lane took a transaction per lane. What a chunk needs besides the accumulator is read before
+//    it, and the accumulator is given back by a relaxed arrive after its last read: a release at cluster scope waited for the
+//    stores of the whole tile (8192 x 3072 x 768 with GELU 63 us, 45 without that wait). 12 or 16 warps leave a ring of 5
+//    stages and too few registers: BERT-base 64 x 128 3.32 -> 3.53 and 3.58 ms, the 2048-token prompt 3.48 -> 3.68.
 //
 // Measured against the one-CTA tiles of 128 rows x 256 or 128 columns (gemm_tc.cu), which loaded 48 KB per k-block and SM (about
 // 68 bytes per clock, the most seen) and ended in a last wave of a few tiles. 2048 rows: 12288 x 4096 144 -> 115 us (1.79
 // PFLOP/s), 22016 x 4096 228 -> 200, 4096 x 11008 143 -> 105, 4096 x 4096 67 -> 50; 680 rows x 8192 x 32768 419 -> 259;
-// 8192 rows x 768 x 768 with residual 36 -> 23. Bound by the tensor cores from K of about 2000 on (0.9 of their rate at the
+// 8192 rows x 768 x 768 with residual 36 -> 22, x 3072 x 768 with GELU 73 -> 45. Bound by the tensor cores from K of about 2000 on (0.9 of their rate at the
 // chosen width), by the epilogue's turn-around and stores below that.
 //
 // CTA = 10 warps: warp 0 lane 0 TMA producer; warp 1 tensor-memory allocator, its lane 0 in CTA 0 issues the pair's MMAs;
@@ -76,8 +79,10 @@ __device__ __forceinline__ uint32_t at_leader(uint32_t local) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(local));
   return r;
 }
+// Relaxed: it tells of accumulator reads (ordered by the tcgen05 fence before it) and of no memory; a release at cluster scope
+// would wait for the warp's result stores.
 __device__ __forceinline__ void arrive_cluster(uint32_t bar) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 // A 2-D box into this CTA's shared memory, completing on a barrier of either CTA of the pair.
 __device__ __forceinline__ void pair_load_2d(const CUtensorMap* tm, uint32_t bar, uint32_t dst, int x, int y) {
@@ -115,76 +120,212 @@ __device__ __forceinline__ bool wait_fixed(uint64_t* bar, uint32_t par, unsigned
 __device__ __forceinline__ float pg_block_cycles(int bn) { return fmaxf(2.f * bn, 205.f + 0.8f * bn); }
 
 // ---------------------------------------------------------------------------- epilogue of one 32 x 32 chunk
-struct PgWarp {
-  const float* stg;   // the warp's staged chunk
-  int lane;
-  int ra0, n_rows;    // GEMM row of the chunk's row 0; rows of the chunk that exist
-};
-// 4 staged values: row r, columns 4 p .. 4 p + 3 (16-byte pieces lie XOR-swizzled by the row)
-__device__ __forceinline__ float4 staged(const float* stg, int r, int p) {
-  return *reinterpret_cast<const float4*>(stg + r * 32 + ((p ^ (r & 7)) << 2));
+// A staged chunk's rows lie one after another, their 16-byte pieces XOR-swizzled so that neither a piece per row (as tensor
+// memory gives them) nor the pieces of whole rows (as they are read back) meet in a bank: fp32 rows of 8 pieces, bf16 rows of
+// 4, SwiGLU's 16 bf16 results in 2.
+__device__ __forceinline__ int piece32(int r, int p) { return r * 128 + ((p ^ (r & 7)) << 4); }
+__device__ __forceinline__ int piece16(int r, int p) { return r * 64 + ((p ^ ((r >> 1) & 3)) << 4); }
+__device__ __forceinline__ int piece8(int r, int p) { return r * 32 + ((p ^ ((r >> 2) & 1)) << 4); }
+__device__ __forceinline__ uint32_t bf16x2(float a, float b) {
+  const __nv_bfloat162 x = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<const uint32_t*>(&x);
 }
-__device__ __forceinline__ uint2 to_bf16x4(float a, float b, float c, float d) {
-  const __nv_bfloat162 x = __floats2bfloat162_rn(a, b), y = __floats2bfloat162_rn(c, d);
-  return make_uint2(*reinterpret_cast<const uint32_t*>(&x), *reinterpret_cast<const uint32_t*>(&y));
-}
-__device__ __forceinline__ void act4(int act, float (&v)[4]) {
-  if (act == ACT_GELU_ERF) {
+// bf_only: the results are rounded to bf16 and kept in no wider type
+__device__ __forceinline__ void act32(int act, bool bf_only, float (&v)[32]) {
+  if (act == ACT_GELU_ERF && bf_only) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) v[j] = gelu_erf_f(v[j]);
-  } else if (act == ACT_GELU_TANH) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float x = v[j], u = 0.79788456080286536f * (x + 0.044715f * x * x * x);
-      v[j] = 0.5f * x * (1.f + tanh_approx(u));
-    }
-  } else if (act == ACT_TANH) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) v[j] = tanhf(v[j]);
+    for (int j = 0; j < 32; ++j) v[j] = gelu_erf_bf(v[j]);
+  } else {
+    act_chunk32<bf16>(act, v);
   }
 }
 
-// Whether the chunk epilogues may move 16-byte (fp32) and 8-byte (bf16) pieces of the operands they use.
+// Whether the chunk epilogues may move 16-byte pieces of the operands they use.
+template <int KIND>
 __device__ __forceinline__ bool pg_vectors(const Epi& e) {
-  switch (e.kind) {
-    case EPI_F32: return ((uintptr_t)e.out_f32 & 15) == 0 && (e.ld_f32 & 3) == 0;
-    case EPI_ACT:
-      return ((uintptr_t)e.out_t & 7) == 0 && (e.ld_t & 3) == 0 &&
-             (!e.out_f32 || (((uintptr_t)e.out_f32 & 15) == 0 && (e.ld_f32 & 3) == 0));
-    case EPI_RESID:
-      return ((uintptr_t)e.out_f32 & 15) == 0 && (e.ld_f32 & 3) == 0 && ((uintptr_t)e.resid & 15) == 0 &&
-             (e.ld_resid & 3) == 0;
-    case EPI_SWIGLU: return ((uintptr_t)e.out_t & 7) == 0 && (e.ld_t & 3) == 0;
-    default: return true;
+  const bool f32 = ((uintptr_t)e.out_f32 & 15) == 0 && (e.ld_f32 & 3) == 0, t = ((uintptr_t)e.out_t & 15) == 0 && (e.ld_t & 7) == 0;
+  switch (KIND) {
+    case EPI_F32: return f32;
+    case EPI_ACT: return t && (!e.out_f32 || f32);
+    case EPI_RESID: return f32 && ((uintptr_t)e.resid & 15) == 0 && (e.ld_resid & 3) == 0;
+    case EPI_SWIGLU: return t;
+    default: return true;   // heads of whole 32-column chunks
   }
 }
 
-// F32 / ACT / RESID chunks with a ragged edge or rows that are not whole pieces: a lane per column, a row at a time.
-__device__ void pg_chunk_scalar(const Epi& e, const PgWarp& w, int c0, int N) {
-  const int c = c0 + w.lane;
-  const float b = (e.bias && c < N) ? e.bias[c] : 0.f;
-#pragma unroll 1
-  for (int r = 0; r < w.n_rows; ++r) {
-    float v = w.stg[r * 32 + (((w.lane >> 2) ^ (r & 7)) << 2) + (w.lane & 3)] + b;
-    if (c >= N) continue;
-    const size_t ra = (size_t)(w.ra0 + r);
-    if (e.kind == EPI_RESID) {
-      e.out_f32[ra * e.ld_f32 + c] = e.resid[ra * e.ld_resid + c] + v;
-    } else if (e.kind == EPI_F32) {
-      e.out_f32[ra * e.ld_f32 + c] = v;
-    } else {
-      if (e.act == ACT_GELU_TANH)
-        v = 0.5f * v * (1.f + tanh_approx(0.79788456080286536f * (v + 0.044715f * v * v * v)));
-      else
-        v = apply_act(e.act, v);
-      ((bf16*)e.out_t)[ra * e.ld_t + c] = from_f<bf16>(v);
-      if (e.out_f32) e.out_f32[ra * e.ld_f32 + c] = v;
+// The epilogue of 32 rows of a tile.
+template <int KIND>
+struct PgTile {
+  const Epi& e;
+  uint8_t* stg;        // the warp's staging chunk
+  int lane, ra0, n_rows, cb, ce, N;   // rows ra0 .., columns cb .. cb + ce
+  bool vec;
+  EpiRow rr;           // cache epilogues: this lane's row
+  // what a chunk reads besides the accumulator
+  struct In {
+    float bias;        // of column `lane`
+    float4 rs[KIND == EPI_RESID ? 8 : 1];
+  };
+
+  __device__ __forceinline__ void load(In& in, int c) const {
+    const int lr = lane >> 3, lp = lane & 7, c0 = cb + c;
+    if (c >= ce) return;
+    in.bias = (e.bias && c0 + lane < N) ? e.bias[c0 + lane] : 0.f;
+    if (KIND == EPI_RESID && vec && c0 + 32 <= N) {
+      const float* src = e.resid + (size_t)(ra0 + lr) * e.ld_resid + c0 + lp * 4;
+      const size_t step = (size_t)4 * e.ld_resid;
+#pragma unroll
+      for (int i = 0; i < 8; ++i, src += step)
+        in.rs[i] = 4 * i + lr < n_rows ? *reinterpret_cast<const float4*>(src) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
   }
-}
+  __device__ __forceinline__ float4 staged32(int r, int p) const { return *reinterpret_cast<const float4*>(stg + piece32(r, p)); }
+  __device__ __forceinline__ void stage32(const float (&v)[32]) const {
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      *reinterpret_cast<float4*>(stg + piece32(lane, k)) = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+    __syncwarp();
+  }
+  __device__ __forceinline__ void stage16(const float (&v)[32]) const {
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      *reinterpret_cast<uint4*>(stg + piece16(lane, k)) =
+          make_uint4(bf16x2(v[8 * k], v[8 * k + 1]), bf16x2(v[8 * k + 2], v[8 * k + 3]), bf16x2(v[8 * k + 4], v[8 * k + 5]),
+                     bf16x2(v[8 * k + 6], v[8 * k + 7]));
+    __syncwarp();
+  }
+  // F32 / ACT / RESID chunks with a ragged edge, or whose rows are not whole pieces: a lane per column, a row at a time.
+  __device__ __forceinline__ void store_columns(int c0) const {
+    const int c = c0 + lane;
+#pragma unroll 1
+    for (int r = 0; r < n_rows; ++r) {
+      const float v = *reinterpret_cast<const float*>(stg + piece32(r, lane >> 2) + (lane & 3) * 4);
+      if (c >= N) continue;
+      const size_t ra = (size_t)(ra0 + r);
+      if (KIND == EPI_ACT) ((bf16*)e.out_t)[ra * e.ld_t + c] = from_f<bf16>(v);
+      if (KIND != EPI_ACT || e.out_f32)
+        e.out_f32[ra * e.ld_f32 + c] = KIND == EPI_RESID ? v + e.resid[ra * e.ld_resid + c] : v;
+    }
+  }
+  // 32 fp32 results per row, with the residual: a row piece of 128 bytes per 8 lanes
+  __device__ __forceinline__ void store32(int c0, const In& in) const {
+    const int lr = lane >> 3, lp = lane & 7;
+    float* o = e.out_f32 + (size_t)(ra0 + lr) * e.ld_f32 + c0 + lp * 4;
+    const size_t step = (size_t)4 * e.ld_f32;
+#pragma unroll
+    for (int i = 0; i < 8; ++i, o += step) {
+      float4 y = staged32(4 * i + lr, lp);
+      if (KIND == EPI_RESID) y = make_float4(y.x + in.rs[i].x, y.y + in.rs[i].y, y.z + in.rs[i].z, y.w + in.rs[i].w);
+      if (4 * i + lr < n_rows) *reinterpret_cast<float4*>(o) = y;
+    }
+  }
+
+  // free: the pair's barrier for this accumulator, told after the warp's last read of it
+  __device__ __forceinline__ void chunk(uint32_t tb, int c, const In& in, uint32_t free, bool last) const {
+    const int c0 = cb + c;
+    float v[32];
+    tmem_ld32(tb + (uint32_t)c, v);
+    tc_fence_before();
+    __syncwarp();   // the chunk before this one has been read
+    if (last && lane == 0) arrive_cluster(free);
+    if (e.bias) {
+      reinterpret_cast<float*>(stg)[lane] = in.bias;
+      __syncwarp();
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const float4 b = reinterpret_cast<const float4*>(stg)[k];
+        v[4 * k] += b.x;
+        v[4 * k + 1] += b.y;
+        v[4 * k + 2] += b.z;
+        v[4 * k + 3] += b.w;
+      }
+      __syncwarp();
+    }
+    if constexpr (KIND == EPI_SWIGLU) {
+      // the row's 16 gate and 16 up columns meet in this lane
+#pragma unroll
+      for (int j = 0; j < 16; ++j) v[j] = silu_f(v[j]) * v[16 + j];
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+        *reinterpret_cast<uint4*>(stg + piece8(lane, k)) =
+            make_uint4(bf16x2(v[8 * k], v[8 * k + 1]), bf16x2(v[8 * k + 2], v[8 * k + 3]), bf16x2(v[8 * k + 4], v[8 * k + 5]),
+                       bf16x2(v[8 * k + 6], v[8 * k + 7]));
+      __syncwarp();
+      const int lr = lane >> 1, lp = lane & 1;
+      bf16* o = (bf16*)e.out_t + (size_t)(ra0 + lr) * e.ld_t + (c0 >> 1) + lp * 8;
+#pragma unroll
+      for (int i = 0; i < 2; ++i, o += (size_t)16 * e.ld_t) {
+        if (16 * i + lr >= n_rows) continue;
+        const uint4 x = *reinterpret_cast<const uint4*>(stg + piece8(16 * i + lr, lp));
+        if (vec) {
+          *reinterpret_cast<uint4*>(o) = x;
+        } else {
+          const bf16* h = reinterpret_cast<const bf16*>(&x);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) o[j] = h[j];
+        }
+      }
+    } else if constexpr (KIND <= EPI_RESID) {
+      if (KIND == EPI_ACT) act32(e.act, e.out_f32 == nullptr, v);
+      const bool whole = vec && c0 + 32 <= N;
+      if (KIND != EPI_ACT || !whole || e.out_f32) {
+        stage32(v);
+        if (!whole) {
+          store_columns(c0);
+          return;
+        }
+        store32(c0, in);
+      }
+      if constexpr (KIND == EPI_ACT) {
+        if (e.out_f32) __syncwarp();
+        stage16(v);
+        const int lr = lane >> 2, lp = lane & 3;
+        bf16* o = (bf16*)e.out_t + (size_t)(ra0 + lr) * e.ld_t + c0 + lp * 8;
+        const size_t step = (size_t)8 * e.ld_t;
+#pragma unroll
+        for (int i = 0; i < 4; ++i, o += step)
+          if (8 * i + lr < n_rows) *reinterpret_cast<uint4*>(o) = *reinterpret_cast<const uint4*>(stg + piece16(8 * i + lr, lp));
+      }
+    } else {
+      // query columns, then key, then value (a chunk lies inside one head of one of them)
+      const int dh = e.head_dim, nq = e.n_q_cols, nkv = e.n_kv_cols, lr = lane >> 2, lp = lane & 3;
+      const bool is_q = c0 < nq, is_k = !is_q && c0 < nq + nkv;
+      const int cc = is_q ? c0 : is_k ? c0 - nq : c0 - nq - nkv, h = cc / dh, d0 = cc - h * dh;
+      bf16* base = is_q ? (bf16*)e.out_t + (size_t)ra0 * e.ld_t + h * dh
+                        : (bf16*)(is_k ? e.cache.k : e.cache.v) + (size_t)h * e.cache.head_stride();
+      const bool rope = e.rope && (is_q || is_k);
+      if (rope)
+        stage32(v);
+      else
+        stage16(v);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int r = 8 * i + lr;
+        long long slot = __shfl_sync(0xffffffffu, rr.cbase, r);
+        const int pos = __shfl_sync(0xffffffffu, rr.pos, r);
+        if (is_q) slot = (long long)r * e.ld_t;
+        if (r >= n_rows || slot < 0) continue;
+        if (rope) {
+          // columns (2 j, 2 j + 1) hold the rotate-half pair (j, j + dh / 2); 4 pairs per lane
+          const int half_d = dh >> 1, j0 = (d0 >> 1) + lp * 4;
+          const float4* tab = reinterpret_cast<const float4*>(e.rope_table + (size_t)pos * half_d + j0);
+          const float4 x = staged32(r, 2 * lp), y = staged32(r, 2 * lp + 1), s = tab[0], t = tab[1];
+          bf16* d = base + slot + j0;
+          const float2 a0 = rope_turn(x.x, x.y, s.x, s.y), a1 = rope_turn(x.z, x.w, s.z, s.w);
+          const float2 a2 = rope_turn(y.x, y.y, t.x, t.y), a3 = rope_turn(y.z, y.w, t.z, t.w);
+          *reinterpret_cast<uint2*>(d) = make_uint2(bf16x2(a0.x, a1.x), bf16x2(a2.x, a3.x));
+          *reinterpret_cast<uint2*>(d + half_d) = make_uint2(bf16x2(a0.y, a1.y), bf16x2(a2.y, a3.y));
+        } else {
+          *reinterpret_cast<uint4*>(base + slot + d0 + lp * 8) = *reinterpret_cast<const uint4*>(stg + piece16(r, lp));
+        }
+      }
+    }
+  }
+};
 
 // ---------------------------------------------------------------------------- kernel
-template <int MAXG>
+// KIND: the epilogue of every problem of the launch (EPI_QKV also for EPI_KV)
+template <int KIND, int MAXG>
 __global__ void __launch_bounds__(PG_THREADS, 1) gemm_pair_kernel(const __grid_constant__ PgParams<MAXG> p) {
   KT_BEGIN();
   extern __shared__ uint8_t pg_smem_raw[];
@@ -367,173 +508,57 @@ __global__ void __launch_bounds__(PG_THREADS, 1) gemm_pair_kernel(const __grid_c
     } else {
       // -------------------------------------------------------------- epilogue warps 2..9
       const int q = warp & 3;              // TMEM lane quarter this warp may access
-      const int half = (warp - 2) >> 2;    // this warp takes the chunks of its parity
-      float* stg = reinterpret_cast<float*>(smem + PG_RING + (warp - 2) * PG_STG);
+      const int part = (warp - 2) >> 2;    // this warp takes every other chunk
+      constexpr int STEP = 32 * (PG_EPI_WARPS / 4);
+      uint8_t* stg = smem + PG_RING + (warp - 2) * PG_STG;
       const uint32_t acce0 = at_leader(smem_u32(acce));
-      const int lr = lane >> 3, lp = lane & 7;   // turned around: row 4 i + lr, 16-byte piece lp
       int ab = 0;
       uint32_t aph = 0;
+      EpiRow rr{-1, 0, nullptr};
+      int tok = -1, seq = 0, pos = 0;   // the next tile's row, one of its three dependent look-ups at a time
       for (int t = pair; t < total; t += n_pairs) {
         int g, mb, nb;
         locate(t, g, mb, nb);
-        const Epi& e = p.g[g].epi;
-        const int N = p.g[g].N, kind = e.kind;
-        const int r0 = mb * PG_BM + rank * 128 + q * 32;   // the warp's first row within the group
-        PgWarp w{stg, lane, s_mbeg[g] + r0, max(0, min(32, s_M[g] - r0))};
-        const bool vec = pg_vectors(e);
-        // a row's cache slot, the first chunk's residual: before the accumulator is there
-        EpiRow rr{-1, 0, nullptr};
-        if (lane < w.n_rows) rr = epi_row(e, w.ra0 + lane);
-        float4 rs[8];
-        auto load_resid = [&](int c0) {
-          if (kind != EPI_RESID || !vec || c0 + 32 > N) return;
-          const float* src = e.resid + (size_t)w.ra0 * e.ld_resid + c0 + lp * 4;
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const int r = 4 * i + lr;
-            rs[i] = r < w.n_rows ? *reinterpret_cast<const float4*>(src + (size_t)r * e.ld_resid) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const Epi e = p.g[g].epi;
+        const int N = p.g[g].N, row0 = rank * 128 + q * 32;
+        const int r0 = mb * PG_BM + row0;   // the warp's first row within the group
+        const int n_rows = max(0, min(32, s_M[g] - r0));
+        int gn = 0;
+        if (KIND == EPI_QKV) {
+          if (t == pair && lane < n_rows) rr = epi_row(e, s_mbeg[g] + r0 + lane);
+          tok = -1;
+          if (t + n_pairs < total) {
+            int m2, n2;
+            locate(t + n_pairs, gn, m2, n2);
+            const int r = m2 * PG_BM + row0 + lane;
+            if (r < s_M[gn]) tok = p.g[gn].epi.row_tok[s_mbeg[gn] + r];
           }
-        };
-        const int cb = nb * BN, ce = min(BN, N - cb);   // the tile's columns
-        load_resid(cb + half * 32);
+        }
+        const PgTile<KIND> tile{e, stg, lane, s_mbeg[g] + r0, n_rows, nb * BN, min(BN, N - nb * BN), N, pg_vectors<KIND>(e), rr};
+        // the first chunk's bias and residual, before the accumulator is there
+        typename PgTile<KIND>::In in;
+        int c = part * 32;
+        tile.load(in, c);
         bool got = true;
         if (lane == 0) got = mbar_wait(&accf[ab], aph, abort_flag, p.err, wlim);
         got = __shfl_sync(0xffffffffu, got ? 1 : 0, 0) != 0;
         if (!got) break;   // warp-uniform: tcgen05.ld below is .sync.aligned
         tc_fence_after();
         const uint32_t tb = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(ab * 256);
-#pragma unroll 1
-        for (int c = half * 32; c < ce; c += 64) {
-          const int c0 = cb + c;
-          float v[32];
-          tmem_ld32(tb + (uint32_t)c, v);
-          if (kind == EPI_SWIGLU) {
-            // the row's 16 gate and 16 up columns meet in this lane
-            if (e.bias) {
-#pragma unroll
-              for (int j = 0; j < 32; ++j) v[j] += e.bias[c0 + j];
-            }
-#pragma unroll
-            for (int j = 0; j < 16; ++j) v[j] = silu_f(v[j]) * v[16 + j];
-          }
-          __syncwarp();   // the chunk before this one has been read
-          float4* row = reinterpret_cast<float4*>(stg + lane * 32);
-          if (kind == EPI_SWIGLU) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-              row[k ^ (lane & 7)] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
-          } else {
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-              row[k ^ (lane & 7)] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
-          }
-          __syncwarp();
-          if (kind == EPI_SWIGLU) {
-            // 16 results per row: 4 lanes of 4
-            bf16* o = (bf16*)e.out_t + (size_t)w.ra0 * e.ld_t + (c0 >> 1) + (lane & 3) * 4;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const int r = 8 * i + (lane >> 2);
-              if (r >= w.n_rows) continue;
-              const float4 x = staged(stg, r, lane & 3);
-              bf16* d = o + (size_t)r * e.ld_t;
-              if (vec) {
-                *reinterpret_cast<uint2*>(d) = to_bf16x4(x.x, x.y, x.z, x.w);
-              } else {
-                d[0] = from_f<bf16>(x.x);
-                d[1] = from_f<bf16>(x.y);
-                d[2] = from_f<bf16>(x.z);
-                d[3] = from_f<bf16>(x.w);
-              }
-            }
-          } else if (kind <= EPI_RESID) {
-            if (!vec || c0 + 32 > N) {
-              pg_chunk_scalar(e, w, c0, N);
-            } else {
-              float4 b4 = make_float4(0.f, 0.f, 0.f, 0.f);
-              if (e.bias) {
-                const float* bp = e.bias + c0 + lp * 4;
-                b4 = make_float4(bp[0], bp[1], bp[2], bp[3]);
-              }
-              if (kind == EPI_ACT) {
-                bf16* o = (bf16*)e.out_t + (size_t)w.ra0 * e.ld_t + c0 + lp * 4;
-                float* f = e.out_f32 ? e.out_f32 + (size_t)w.ra0 * e.ld_f32 + c0 + lp * 4 : nullptr;
-#pragma unroll 2
-                for (int i = 0; i < 8; ++i) {
-                  const int r = 4 * i + lr;
-                  const float4 x = staged(stg, r, lp);
-                  float y[4] = {x.x + b4.x, x.y + b4.y, x.z + b4.z, x.w + b4.w};
-                  act4(e.act, y);
-                  if (r < w.n_rows) {
-                    *reinterpret_cast<uint2*>(o + (size_t)r * e.ld_t) = to_bf16x4(y[0], y[1], y[2], y[3]);
-                    if (f) *reinterpret_cast<float4*>(f + (size_t)r * e.ld_f32) = make_float4(y[0], y[1], y[2], y[3]);
-                  }
-                }
-              } else {
-                float* o = e.out_f32 + (size_t)w.ra0 * e.ld_f32 + c0 + lp * 4;
-                if (kind == EPI_RESID) {
-#pragma unroll
-                  for (int i = 0; i < 8; ++i) {
-                    const int r = 4 * i + lr;
-                    const float4 x = staged(stg, r, lp);
-                    if (r < w.n_rows)
-                      *reinterpret_cast<float4*>(o + (size_t)r * e.ld_f32) =
-                          make_float4((x.x + b4.x) + rs[i].x, (x.y + b4.y) + rs[i].y, (x.z + b4.z) + rs[i].z,
-                                      (x.w + b4.w) + rs[i].w);
-                  }
-                  load_resid(c0 + 64);
-                } else {
-#pragma unroll
-                  for (int i = 0; i < 8; ++i) {
-                    const int r = 4 * i + lr;
-                    const float4 x = staged(stg, r, lp);
-                    if (r < w.n_rows)
-                      *reinterpret_cast<float4*>(o + (size_t)r * e.ld_f32) =
-                          make_float4(x.x + b4.x, x.y + b4.y, x.z + b4.z, x.w + b4.w);
-                  }
-                }
-              }
-            }
-          } else {
-            // query columns, then key, then value (a chunk lies inside one head of one of them)
-            const int dh = e.head_dim, nq = e.n_q_cols, nkv = e.n_kv_cols;
-            const bool is_q = c0 < nq, is_k = !is_q && c0 < nq + nkv;
-            const int cc = is_q ? c0 : is_k ? c0 - nq : c0 - nq - nkv, h = cc / dh, d0 = cc - h * dh;
-            const bool rope = e.rope && (is_q || is_k);
-            bf16* base = is_q ? (bf16*)e.out_t + (size_t)w.ra0 * e.ld_t + h * dh
-                              : (bf16*)(is_k ? e.cache.k : e.cache.v) + (size_t)h * e.cache.head_stride();
-            float4 b4 = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (e.bias) {
-              const float* bp = e.bias + c0 + lp * 4;
-              b4 = make_float4(bp[0], bp[1], bp[2], bp[3]);
-            }
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const int r = 4 * i + lr;
-              const long long slot = __shfl_sync(0xffffffffu, rr.cbase, r);
-              const int pos = __shfl_sync(0xffffffffu, rr.pos, r);
-              float4 x = staged(stg, r, lp);
-              x = make_float4(x.x + b4.x, x.y + b4.y, x.z + b4.z, x.w + b4.w);
-              if (r >= w.n_rows || (!is_q && slot < 0)) continue;
-              bf16* d = is_q ? base + (size_t)r * e.ld_t : base + slot;
-              if (rope) {
-                // columns (2 j, 2 j + 1) hold the rotate-half pair (j, j + dh / 2)
-                const int half_d = dh >> 1, j0 = (d0 >> 1) + lp * 2;
-                const float2* tab = e.rope_table + (size_t)pos * half_d + j0;
-                const float2 u = tab[0], z = tab[1];
-                *reinterpret_cast<__nv_bfloat162*>(d + j0) =
-                    __floats2bfloat162_rn(x.x * u.x - x.y * u.y, x.z * z.x - x.w * z.y);
-                *reinterpret_cast<__nv_bfloat162*>(d + j0 + half_d) =
-                    __floats2bfloat162_rn(x.y * u.x + x.x * u.y, x.w * z.x + x.z * z.y);
-              } else {
-                *reinterpret_cast<uint2*>(d + d0 + lp * 4) = to_bf16x4(x.x, x.y, x.z, x.w);
-              }
-            }
-          }
+        if (KIND == EPI_QKV && tok >= 0) {
+          seq = p.g[gn].epi.tok_seq[tok];
+          pos = p.g[gn].epi.tok_pos[tok];
         }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) arrive_cluster(acce0 + (uint32_t)ab * 8);
+#pragma unroll 1
+        for (; c < tile.ce; c += STEP) {
+          tile.chunk(tb, c, in, acce0 + (uint32_t)ab * 8, c + STEP >= tile.ce);
+          tile.load(in, c + STEP);
+        }
+        if (KIND == EPI_QKV) {
+          rr.cbase = tok >= 0 ? p.g[gn].epi.cache.checked_base(p.g[gn].epi.layer0, seq, pos) : -1;
+          rr.pos = pos;
+        }
+        if (part * 32 >= tile.ce && lane == 0) arrive_cluster(acce0 + (uint32_t)ab * 8);   // no chunk of this tile
         ab ^= 1;
         if (ab == 0) aph ^= 1;
       }
@@ -558,7 +583,7 @@ __global__ void __launch_bounds__(PG_THREADS, 1) gemm_pair_kernel(const __grid_c
 // room for the weight slabs and the output stream.
 int pg_raster(int K) { return (int)std::max(1LL, std::min(32LL, (48LL << 20) / std::max(256LL * K * 2, 1LL))); }
 
-template <int MAXG>
+template <int KIND, int MAXG>
 int pg_pairs() {
   // CTA pairs that are resident at once, 0 when the kernel cannot run
   static int pairs = 0;
@@ -567,7 +592,7 @@ int pg_pairs() {
     int dev = 0, sms = 0, n = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaFuncSetAttribute(gemm_pair_kernel<MAXG>, cudaFuncAttributeMaxDynamicSharedMemorySize, PG_SMEM) != cudaSuccess) {
+    if (cudaFuncSetAttribute(gemm_pair_kernel<KIND, MAXG>, cudaFuncAttributeMaxDynamicSharedMemorySize, PG_SMEM) != cudaSuccess) {
       cudaGetLastError();
       return;
     }
@@ -581,7 +606,7 @@ int pg_pairs() {
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&n, gemm_pair_kernel<MAXG>, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, gemm_pair_kernel<KIND, MAXG>, &cfg) != cudaSuccess) {
       cudaGetLastError();
       return;
     }
@@ -590,9 +615,9 @@ int pg_pairs() {
   return pairs;
 }
 
-template <int MAXG>
+template <int KIND, int MAXG>
 int pg_go(cudaStream_t st, const GemmProblem* probs, int n, unsigned* err) {
-  const int pairs = pg_pairs<MAXG>();
+  const int pairs = pg_pairs<KIND, MAXG>();
   if (pairs <= 0) return -1;
   thread_local PgParams<MAXG> prm;   // one per host thread
   memset(&prm, 0, sizeof prm);
@@ -625,7 +650,7 @@ int pg_go(cudaStream_t st, const GemmProblem* probs, int n, unsigned* err) {
   at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = g_pdl ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, gemm_pair_kernel<MAXG>, prm) == cudaSuccess ? 1 : -1;
+  return cudaLaunchKernelEx(&cfg, gemm_pair_kernel<KIND, MAXG>, prm) == cudaSuccess ? 1 : -1;
 }
 
 }  // namespace
@@ -641,9 +666,24 @@ bool pair_gemm_supported(const GemmProblem& q, int max_rows) {
 
 int pair_gemm(cudaStream_t st, const GemmProblem* probs, int n_probs, const int* max_rows, unsigned* err) {
   if (n_probs < 1 || n_probs > PG_MAXG) return -1;
+  auto kind_of = [](const GemmProblem& q) { return q.epi.kind == EPI_KV ? (int)EPI_QKV : q.epi.kind; };
+  const int kind = kind_of(probs[0]);
   for (int i = 0; i < n_probs; ++i)
-    if (!pair_gemm_supported(probs[i], max_rows[i])) return -1;
-  return n_probs <= 2 ? pg_go<2>(st, probs, n_probs, err) : pg_go<PG_MAXG>(st, probs, n_probs, err);
+    if (!pair_gemm_supported(probs[i], max_rows[i]) || kind_of(probs[i]) != kind) return -1;
+  if (n_probs > 2) {
+    switch (kind) {
+      case EPI_F32: return pg_go<EPI_F32, PG_MAXG>(st, probs, n_probs, err);
+      case EPI_QKV: return pg_go<EPI_QKV, PG_MAXG>(st, probs, n_probs, err);
+      default: return -1;
+    }
+  }
+  switch (kind) {
+    case EPI_F32: return pg_go<EPI_F32, 2>(st, probs, n_probs, err);
+    case EPI_ACT: return pg_go<EPI_ACT, 2>(st, probs, n_probs, err);
+    case EPI_RESID: return pg_go<EPI_RESID, 2>(st, probs, n_probs, err);
+    case EPI_SWIGLU: return pg_go<EPI_SWIGLU, 2>(st, probs, n_probs, err);
+    default: return pg_go<EPI_QKV, 2>(st, probs, n_probs, err);
+  }
 }
 
 ADEPT_KTRACE_ATTACH(pg)
