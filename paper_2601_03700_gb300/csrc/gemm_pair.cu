@@ -147,7 +147,7 @@ __device__ __forceinline__ bool pg_vectors(const Epi& e) {
   switch (KIND) {
     case EPI_F32: return f32;
     case EPI_ACT: return t && (!e.out_f32 || f32);
-    case EPI_RESID: return f32 && ((uintptr_t)e.resid & 15) == 0 && (e.ld_resid & 3) == 0;
+    case EPI_RESID: return f32 && (!e.resid || (((uintptr_t)e.resid & 15) == 0 && (e.ld_resid & 3) == 0));
     case EPI_SWIGLU: return t;
     default: return true;   // heads of whole 32-column chunks
   }
@@ -171,7 +171,10 @@ struct PgTile {
     const int lr = lane >> 3, lp = lane & 7, c0 = cb + c;
     if (c >= ce) return;
     in.bias = (e.bias && c0 + lane < N) ? e.bias[c0 + lane] : 0.f;
-    if (KIND == EPI_RESID && vec && c0 + 32 <= N) {
+    if (KIND == EPI_RESID && !e.resid) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) in.rs[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    } else if (KIND == EPI_RESID && vec && c0 + 32 <= N) {
       const float* src = e.resid + (size_t)(ra0 + lr) * e.ld_resid + c0 + lp * 4;
       const size_t step = (size_t)4 * e.ld_resid;
 #pragma unroll
@@ -204,7 +207,7 @@ struct PgTile {
       const size_t ra = (size_t)(ra0 + r);
       if (KIND == EPI_ACT) ((bf16*)e.out_t)[ra * e.ld_t + c] = from_f<bf16>(v);
       if (KIND != EPI_ACT || e.out_f32)
-        e.out_f32[ra * e.ld_f32 + c] = KIND == EPI_RESID ? v + e.resid[ra * e.ld_resid + c] : v;
+        e.out_f32[ra * e.ld_f32 + c] = KIND == EPI_RESID && e.resid ? v + e.resid[ra * e.ld_resid + c] : v;
     }
   }
   // 32 fp32 results per row, with the residual: a row piece of 128 bytes per 8 lanes
@@ -324,7 +327,7 @@ struct PgTile {
 };
 
 // ---------------------------------------------------------------------------- kernel
-// KIND: the epilogue of every problem of the launch (EPI_QKV also for EPI_KV)
+// KIND: the epilogue of every problem of the launch (EPI_QKV also for EPI_KV, EPI_RESID also for EPI_F32)
 template <int KIND, int MAXG>
 __global__ void __launch_bounds__(PG_THREADS, 1) gemm_pair_kernel(const __grid_constant__ PgParams<MAXG> p) {
   KT_BEGIN();
@@ -666,10 +669,16 @@ bool pair_gemm_supported(const GemmProblem& q, int max_rows) {
 
 int pair_gemm(cudaStream_t st, const GemmProblem* probs, int n_probs, const int* max_rows, unsigned* err) {
   if (n_probs < 1 || n_probs > PG_MAXG) return -1;
+  // one kernel for EPI_QKV and EPI_KV problems, and one for EPI_F32 and EPI_RESID ones (those without a residual)
   auto kind_of = [](const GemmProblem& q) { return q.epi.kind == EPI_KV ? (int)EPI_QKV : q.epi.kind; };
-  const int kind = kind_of(probs[0]);
-  for (int i = 0; i < n_probs; ++i)
-    if (!pair_gemm_supported(probs[i], max_rows[i]) || kind_of(probs[i]) != kind) return -1;
+  int kind = kind_of(probs[0]);
+  for (int i = 0; i < n_probs; ++i) {
+    if (!pair_gemm_supported(probs[i], max_rows[i])) return -1;
+    const int k = kind_of(probs[i]);
+    if (k == kind) continue;
+    if ((k != EPI_F32 && k != EPI_RESID) || (kind != EPI_F32 && kind != EPI_RESID)) return -1;
+    kind = EPI_RESID;
+  }
   if (n_probs > 2) {
     switch (kind) {
       case EPI_F32: return pg_go<EPI_F32, PG_MAXG>(st, probs, n_probs, err);
