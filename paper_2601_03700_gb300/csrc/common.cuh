@@ -271,11 +271,17 @@ __device__ __forceinline__ float gelu_erf_f(float x) { return 0.5f * x * (1.f + 
 // instructions where erff takes about 60. Against 64 bits: 3.4e-8 of the result's norm over N(0, 1) and 1.0e-7 over
 // N(0, 0.1), the erff form 3.8e-8 in both; the rounding to bf16 is 1.7e-3. Below -3 it keeps 6 digits, the erff form 1.
 // NaN and the infinities as the erff form gives them.
-__device__ __forceinline__ float gelu_erf_bf(float x) {
-  const float z = fminf(fabsf(x), 20.f), d = fmaf(0.33f, z, 1.f), a = z * (z * -0.72134752044448170f);
-  float t, e;
+__device__ __forceinline__ float ex2_approx(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+// R(t) for z = min(|x|, 20); e = exp(-z^2 / 2).
+__device__ __forceinline__ float normal_tail(float z, float& e) {
+  const float d = fmaf(0.33f, z, 1.f);
+  float t;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(d));
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(a));
+  e = ex2_approx(z * (z * -0.72134752044448170f));
   float r = 0.04947014978f;
   r = fmaf(r, t, -0.23992625065f);
   r = fmaf(r, t, 0.37131077812f);
@@ -283,7 +289,12 @@ __device__ __forceinline__ float gelu_erf_bf(float x) {
   r = fmaf(r, t, 0.21082835485f);
   r = fmaf(r, t, 0.10797602751f);
   r = fmaf(r, t, 0.13499328363f);
-  r = fmaf(r, t, -0.00020231069264f);
+  return fmaf(r, t, -0.00020231069264f);
+}
+__device__ __forceinline__ float gelu_erf_bf(float x) {
+  const float z = fminf(fabsf(x), 20.f);
+  float e;
+  const float r = normal_tail(z, e);
   return fmaf(0.5f, fabsf(x), 0.5f * x) - z * e * r;
 }
 __device__ __forceinline__ float gelu_tanh_f(float x) {

@@ -68,7 +68,7 @@ void ht_launch_out_bwd(cudaStream_t st, int dt, const float* dxh, int nsplit, si
 void ht_launch_mid_bwd(cudaStream_t st, int dt, const float* dh4, const float* h3, int n, int m1, const float* g1,
                        float eps, float* dh3f, void* dh3t, float* r1);
 // GELU (bwd = 0: h = GELU(z) into hf (optional), ht, hT) or its derivative (bwd = 1: dz = hf *
-// GELU'(z) in place in hf, and into ht, hT), with the transposed copy hT [C][ldT] (zero columns
+// GELU'(z) into ht, hT), with the transposed copy hT [C][ldT] (zero columns
 // n..ldT-1) written by the same launch.
 // bwd = 1 also leaves the chunk partials of the column sums of dz in part ([chunks(n)][C], for
 // ht_launch_colsum_finish).

@@ -4,6 +4,7 @@
 #define ADEPT_TU_ID 10
 #include "common.cuh"
 #include "kernels.h"
+#include "row_group.cuh"
 
 #include <algorithm>
 
@@ -14,49 +15,6 @@ namespace adept {
 // the first reduction, by a group of TPR threads: a warp for rows of up to 1024 elements (no
 // barrier in the reduction, eight rows per CTA), the whole CTA of 256 above.  V = 0: rows of more
 // than 8192 elements, which are read again from memory after the reduction.
-constexpr int RW_THREADS = 256;
-
-template <int TPR, int NV>
-__device__ __forceinline__ void group_sum(float (&v)[NV], float* red) {
-#pragma unroll
-  for (int i = 0; i < NV; ++i) v[i] = warp_sum(v[i]);
-  if (TPR == 32) return;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  __syncthreads();   // red may still be read by the previous sum
-  if (lane == 0) {
-#pragma unroll
-    for (int i = 0; i < NV; ++i) red[w * NV + i] = v[i];
-  }
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < NV; ++i) {
-    float t = 0.f;
-#pragma unroll
-    for (int k = 0; k < RW_THREADS / 32; ++k) t += red[k * NV + i];
-    v[i] = t;
-  }
-}
-
-// Four elements of a row; `vec`: the row's address allows one 16-byte load.
-__device__ __forceinline__ float4 row4(const float* x, int v, bool vec) {
-  if (vec) return reinterpret_cast<const float4*>(x)[v];
-  return make_float4(x[4 * v], x[4 * v + 1], x[4 * v + 2], x[4 * v + 3]);
-}
-__device__ __forceinline__ void put4(float* o, int v, float4 a) { reinterpret_cast<float4*>(o)[v] = a; }
-__device__ __forceinline__ void put4(bf16* o, int v, float4 a) {
-  const __nv_bfloat162 lo = __floats2bfloat162_rn(a.x, a.y), hi = __floats2bfloat162_rn(a.z, a.w);
-  uint2 u;
-  u.x = *reinterpret_cast<const uint32_t*>(&lo);
-  u.y = *reinterpret_cast<const uint32_t*>(&hi);
-  reinterpret_cast<uint2*>(o)[v] = u;
-}
-__device__ __forceinline__ float sum4(float4 a) { return (a.x + a.y) + (a.z + a.w); }
-__device__ __forceinline__ float dot4(float4 a, float4 b) { return (a.x * b.x + a.y * b.y) + (a.z * b.z + a.w * b.w); }
-__device__ __forceinline__ float4 centre4(float4 a, float mu) {
-  return make_float4(a.x - mu, a.y - mu, a.z - mu, a.w - mu);
-}
-__device__ __forceinline__ float4 scale4(float4 a, float s) { return make_float4(a.x * s, a.y * s, a.z * s, a.w * s); }
-
 // (mean, 1 / deviation) of a row for the attention input of the family: two passes over the
 // held row (the mean first), as the definition reads.  NORM_COPY: (0, 1).
 template <int TPR, int V>
