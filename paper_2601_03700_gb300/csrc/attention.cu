@@ -945,7 +945,7 @@ void launch_attention(cudaStream_t st, int dt, const void* q, int ld_q, void* ou
   // encoder's stop-entirely variant)
   if (decode_keys == 0 && dt == 1 && !key_exit && q_rows > 0 && n_layers > 0 &&
       launch_attention_tc(st, q, ld_q, q_rows, out, ld_out, rows, max_rows, row_tok, tok_seq, tok_pos, seq_len, cache,
-                          n_layers, layer0, n_heads, causal, scale_log2, err) >= 0)
+                          n_layers, layer0, n_heads, causal, scale_log2, kp_len, err) >= 0)
     return;
   if (decode_keys > 0 && ws && counters && dt == 1 && (dh == 64 || dh == 128) && cache.block_tokens == 16 &&
       (decode_keys + AD_CHUNK - 1) / AD_CHUNK <= ATTN_MAX_SPLIT && n_heads % cache.n_kv_heads == 0 &&

@@ -1,7 +1,7 @@
 // Prompt-pass attention on the tcgen05 tensor cores (sm_103a) over the paged KV cache.
 //
-// CTA = one tile of 128 active query rows x one head; 8 warps:
-//   warps 0, 2      TMA producers: the Q tile once (2-D box of the pass's Q rows) and per
+// CTA = one tile of 128 active query rows x one or, for heads of 64, several heads in turn; 12 warps:
+//   warps 0, 2      TMA producers: the Q tile per head (2-D box of the pass's Q rows) and per
 //                   128-key tile the sequence's 8 cache blocks of K (warp 0) and of V (warp 2)
 //                   (one 16-row box per block and 64-wide half of the head), two stages each
 //   warp 1          tensor-memory allocator; lane 0 issues S = Q K^T (M 128, N 128 keys, K d_h,
@@ -13,12 +13,20 @@
 //                   online softmax in the exp2 domain (row maxima exchanged between the two),
 //                   P rounded to bf16 into tensor memory; at the end O / l to the output, half
 //                   of the columns each
-// Tensor memory (512 columns): S 0-255 (two buffers), O 256-383, P 384-511 (two buffers).
+// Tensor memory (512 columns): S 0-255 (two buffers), O 256-383 (heads of 64: two buffers), P 384-511
+// (two buffers).
 // The running maximum of a row is raised only when a tile's maximum exceeds it by more than
 // 2^8 (then the row of O is rescaled in TMEM); below that the probabilities stay <= 2^8, which
 // bf16 and the fp32 accumulator carry exactly as well, and O / l is the same softmax.
 // A tile of rows may span several sequences (rows are in sequence order): the key tiles of
 // each sequence's run are processed in turn, the other rows' probabilities are zero there.
+// Work: a CTA is a chain of latencies (row look-ups, cache blocks, copies, S, softmax, O: 7 to 8 us for
+// one key tile), one CTA per SM. The kernel splits the pass by the rows that are live:
+//  * more (tile, head) pairs than SMs: heads of 64 are taken several per CTA (at_heads), whose copies and
+//    S run ahead of the softmax across heads; the look-ups are paid once;
+//  * few pairs whose tiles span many short sequences: the sequences of a tile are dealt out to up to
+//    AT_MAX_Z CTAs (the launch's z), each computing and writing its own sequences' rows;
+//  * the longest tiles (last rows of causal prompts) start first, all heads of a tile together.
 // Every mbarrier wait is bounded (the runtime wait limit); on time-out the CTA sets the error
 // word, stops, drains its MMAs and copies and frees its tensor memory.
 #define ADEPT_TU_ID 6
@@ -28,6 +36,8 @@
 
 #include <cuda.h>
 
+#include <algorithm>
+
 namespace adept {
 namespace {
 
@@ -35,6 +45,7 @@ constexpr int AT_BM = 128;        // query rows per CTA
 constexpr int AT_BN = 128;        // keys per tile
 constexpr int AT_THREADS = 384;   // K producer, MMA, V producer, idle, 8 softmax warps (two per row)
 constexpr int AT_MAX_SEG = 128;
+constexpr int AT_MAX_Z = 16;
 constexpr float AT_RESCALE_LOG2 = 8.f;   // raise the running maximum only beyond 2^8
 constexpr long long AT_DRAIN_CYCLES = 4000000000LL;
 
@@ -44,7 +55,8 @@ struct AtLayout {
   static constexpr int Q_BYTES = HALVES * AT_BM * 128;    // [half][row][128 B]
   static constexpr int KV_BYTES = HALVES * AT_BN * 128;   // one K or V stage: [half][key][128 B]
   static constexpr int OFF_Q = 0;
-  static constexpr int OFF_K = OFF_Q + Q_BYTES;
+  static constexpr int QB = DH == 64 ? 2 : 1;             // Q buffers (and O buffers): heads in turn
+  static constexpr int OFF_K = OFF_Q + QB * Q_BYTES;
   static constexpr int OFF_V = OFF_K + 2 * KV_BYTES;
   static constexpr int TOTAL = OFF_V + 2 * KV_BYTES;
 };
@@ -63,6 +75,7 @@ struct AtParams {
   const int* block_table;
   int max_blocks_per_seq, n_blocks, n_kv_heads, block_tokens;
   int layer0, n_heads, causal;
+  int z, sms;         // CTAs per (tile, head); SMs
   float scale_log2;
   unsigned* err;
 };
@@ -141,12 +154,6 @@ __device__ __forceinline__ void tmem_st32u(uint32_t taddr, const uint32_t (&v)[3
       "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31])
       : "memory");
 }
-// 2^x by the hardware approximation (relative error ~2^-22; 0 for -inf): one instruction.
-__device__ __forceinline__ float ex2_approx(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
 
 // Non-blocking probe of a phase (try_wait may suspend the thread for a while; a loop that
 // watches several barriers must not sit in one of them).
@@ -166,17 +173,33 @@ __device__ __forceinline__ bool at_wait_warp(uint64_t* bar, uint32_t parity, vol
   return __all_sync(0xffffffffu, ok) != 0;
 }
 
+// Heads per CTA for `tiles` live row tiles: the divisor of n_heads whose rounds over the SMs take the least time, at about 3.5 us
+// of look-ups and set-up per CTA and 2.3 per head.
+__device__ __forceinline__ int at_heads(int tiles, int n_heads, int sms) {
+  int best = 1, best_t = 0x7fffffff;
+  for (int d = 1; d <= n_heads; ++d) {
+    if (n_heads % d) continue;
+    const int t = ((tiles * (n_heads / d) + sms - 1) / sms) * (35 + 23 * d);
+    if (t < best_t) {
+      best = d;
+      best_t = t;
+    }
+  }
+  return best;
+}
+
 template <int DH>
 __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_constant__ AtParams p) {
   using L = AtLayout<DH>;
   extern __shared__ __align__(1024) uint8_t at_raw[];
-  __shared__ __align__(8) uint64_t q_full, k_full[2], v_full[2], k_empty[2], v_empty[2], s_full[2], s_free[2],
+  constexpr int QB = L::QB;
+  __shared__ __align__(8) uint64_t q_full[2], q_free[2], o_free[2], k_full[2], v_full[2], k_empty[2], v_empty[2], s_full[2], s_free[2],
       p_full[2], pv_done[2], drain;
   __shared__ __align__(8) uint64_t pair_bar[4];   // the two softmax warps of a row quarter
   __shared__ float s_xch[2][2][AT_BM];              // their exchanged row maxima / sums
   __shared__ uint32_t s_tmem;
   __shared__ int s_abort;
-  __shared__ int s_rseq[AT_BM], s_rpos[AT_BM];
+  __shared__ int s_rseq[AT_BM], s_rpos[AT_BM], s_rrun[AT_BM];
   __shared__ int s_seg_sq[AT_MAX_SEG], s_seg_kend[AT_MAX_SEG];
   __shared__ int s_nseg, s_nit;
 
@@ -187,12 +210,13 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
   uint8_t* sQ = sm + L::OFF_Q;
   uint8_t* sK = sm + L::OFF_K;
   uint8_t* sV = sm + L::OFF_V;
-  const int h = blockIdx.y, kvh = h / (p.n_heads / p.n_kv_heads);
-  const int tile = (int)gridDim.x - 1 - (int)blockIdx.x;   // late (long causal) tiles start first
+  const int hgroup = p.n_heads / p.n_kv_heads;
 
   if (tid == 0) {
-    mbar_init(&q_full, 1);
     for (int s = 0; s < 2; ++s) {
+      mbar_init(&q_full[s], 1);
+      mbar_init(&q_free[s], 1);
+      mbar_init(&o_free[s], 8);
       mbar_init(&k_full[s], 1);
       mbar_init(&v_full[s], 1);
       mbar_init(&k_empty[s], 1);
@@ -211,8 +235,14 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
   }
   pdl_wait();   // Q rows, row maps and the cache come from the preceding kernels
   pdl_launch_dependents();
-  const int r0 = p.rows.b() + tile * AT_BM, rend = p.rows.e();
-  if (r0 >= rend) return;   // uniform: no rows for this tile
+  // this CTA's tile, heads h0 .. h0 + nh and sequences z, z + Z, ..
+  const int rbeg = p.rows.b(), rend = p.rows.e();
+  const int tiles = (max(0, rend - rbeg) + AT_BM - 1) / AT_BM, Z = p.z;
+  const int nh = QB > 1 && Z == 1 ? at_heads(tiles, p.n_heads, p.sms) : 1;
+  const int per_tile = p.n_heads / nh * Z, id = (int)blockIdx.x;
+  if (id >= tiles * per_tile) return;   // uniform: no work for this CTA
+  const int back = id / per_tile, h0 = (id % per_tile) / Z * nh, z = id % Z;
+  const int r0 = rbeg + (tiles - 1 - back) * AT_BM;   // late (long causal) tiles start first
 
   // rows of the tile: sequence and position (sequence -1 past the active range)
   if (tid < AT_BM) {
@@ -250,6 +280,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
     int before = 0;
     for (int w = 0; w < warp; ++w) before += s_wfirst[w];
     g_row = before + __popc(bal & ((2u << lane) - 1u)) - 1;
+    s_rrun[tid] = g_row;
     if (first) {
       s_seg_sq[g_row] = s_rseq[tid];
       s_seg_kend[g_row] = 0;
@@ -265,13 +296,13 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
   __syncthreads();
   if (warp == 0) {
     int n = 0;
-    for (int g = lane; g < s_nseg; g += 32) n += (s_seg_kend[g] + AT_BN - 1) / AT_BN;
+    for (int g = z + lane * Z; g < s_nseg; g += 32 * Z) n += (s_seg_kend[g] + AT_BN - 1) / AT_BN;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
     if (lane == 0) s_nit = n;
   }
   __syncthreads();
-  const int nseg = s_nseg, nit = s_nit;
+  const int nseg = s_nseg, nit = s_nit;   // key tiles of a head
   const uint32_t tmem = s_tmem;
 
   if (warp == 0 || warp == 2) {
@@ -283,50 +314,59 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
     uint64_t* empty = kw ? k_empty : v_empty;
     const CUtensorMap* map = kw ? &p.kmap : &p.vmap;
     uint8_t* dst0 = kw ? sK : sV;
-    int issued = 0;
+    int issued = 0, q_issued = 0;
     bool ok = true;
-    if (kw && elect_one()) {
-      mbar_expect_tx(&q_full, (uint32_t)L::Q_BYTES);
-      for (int hf = 0; hf < L::HALVES; ++hf) tma_load_2d(&p.qmap, &q_full, sQ + hf * AT_BM * 128, h * DH + hf * 64, r0);
-    }
     int it = 0;
-    for (int g = 0; g < nseg && ok; ++g) {
-      const int sq = s_seg_sq[g], kend = s_seg_kend[g];
-      const int nt = (kend + AT_BN - 1) / AT_BN, nbv = (kend + 15) / 16;
-      const int* bt = p.block_table + (size_t)sq * p.max_blocks_per_seq;
-      for (int j = 0; j < nt && ok; ++j, ++it) {
-        const int s = it & 1;
-        int myrow = 0;
-        if (lane < AT_BN / 16) {
-          // blocks past the run's last key load the last block again (finite values; their
-          // keys are masked and their V rows zeroed before use)
-          int blk = bt[min(j * (AT_BN / 16) + lane, nbv - 1)];
-          if (blk < 0 || blk >= p.n_blocks) {
-            if (kw) atomicOr(p.err, ERRW_POS);
-            blk = 0;
-          }
-          myrow = ((p.layer0 * p.n_blocks + blk) * p.n_kv_heads + kvh) * 16;
-        }
-        int rows8[AT_BN / 16];
-#pragma unroll
-        for (int b = 0; b < AT_BN / 16; ++b) rows8[b] = __shfl_sync(0xffffffffu, myrow, b);
-        if (it >= 2 && !(ok = at_wait_warp(&empty[s], (uint32_t)(((it >> 1) - 1) & 1), abort_flag, p.err, wlim)))
-          break;
+    for (int hh = 0; hh < nh && ok; ++hh) {
+      const int kvh = (h0 + hh) / hgroup;
+      if (kw) {
+        if (hh >= QB && !(ok = at_wait_warp(&q_free[hh % QB], (uint32_t)((hh / QB - 1) & 1), abort_flag, p.err, wlim))) break;
         if (elect_one()) {
-          mbar_expect_tx(&full[s], (uint32_t)L::KV_BYTES);
-          for (int b = 0; b < AT_BN / 16; ++b)
-            for (int hf = 0; hf < L::HALVES; ++hf)
-              tma_load_2d(map, &full[s], dst0 + s * L::KV_BYTES + hf * AT_BN * 128 + b * 16 * 128, hf * 64, rows8[b]);
+          mbar_expect_tx(&q_full[hh % QB], (uint32_t)L::Q_BYTES);
+          for (int hf = 0; hf < L::HALVES; ++hf)
+            tma_load_2d(&p.qmap, &q_full[hh % QB], sQ + hh % QB * L::Q_BYTES + hf * AT_BM * 128, (h0 + hh) * DH + hf * 64, r0);
         }
         __syncwarp();
-        issued = it + 1;
+        q_issued = hh + 1;
+      }
+      for (int g = z; g < nseg && ok; g += Z) {
+        const int sq = s_seg_sq[g], kend = s_seg_kend[g];
+        const int nt = (kend + AT_BN - 1) / AT_BN, nbv = (kend + 15) / 16;
+        const int* bt = p.block_table + (size_t)sq * p.max_blocks_per_seq;
+        for (int j = 0; j < nt && ok; ++j, ++it) {
+          const int s = it & 1;
+          int myrow = 0;
+          if (lane < AT_BN / 16) {
+            // blocks past the run's last key load the last block again (finite values; their
+            // keys are masked and their V rows zeroed before use)
+            int blk = bt[min(j * (AT_BN / 16) + lane, nbv - 1)];
+            if (blk < 0 || blk >= p.n_blocks) {
+              if (kw) atomicOr(p.err, ERRW_POS);
+              blk = 0;
+            }
+            myrow = ((p.layer0 * p.n_blocks + blk) * p.n_kv_heads + kvh) * 16;
+          }
+          int rows8[AT_BN / 16];
+#pragma unroll
+          for (int b = 0; b < AT_BN / 16; ++b) rows8[b] = __shfl_sync(0xffffffffu, myrow, b);
+          if (it >= 2 && !(ok = at_wait_warp(&empty[s], (uint32_t)(((it >> 1) - 1) & 1), abort_flag, p.err, wlim)))
+            break;
+          if (elect_one()) {
+            mbar_expect_tx(&full[s], (uint32_t)L::KV_BYTES);
+            for (int b = 0; b < AT_BN / 16; ++b)
+              for (int hf = 0; hf < L::HALVES; ++hf)
+                tma_load_2d(map, &full[s], dst0 + s * L::KV_BYTES + hf * AT_BN * 128 + b * 16 * 128, hf * 64, rows8[b]);
+          }
+          __syncwarp();
+          issued = it + 1;
+        }
       }
     }
     // every copy issued has landed before the CTA ends (at most the last two tiles are open)
     if (lane == 0) {
-      if (kw) {
+      for (int t = max(0, q_issued - QB); t < q_issued; ++t) {
         const long long tq = clock64();
-        while (!mbar_try_wait(&q_full, 0) && clock64() - tq < AT_DRAIN_CYCLES) {
+        while (!mbar_try_wait(&q_full[t % QB], (uint32_t)((t / QB) & 1)) && clock64() - tq < AT_DRAIN_CYCLES) {
         }
       }
       for (int t = max(0, issued - 2); t < issued; ++t) {
@@ -342,49 +382,62 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
     constexpr uint32_t IDESC_S = at_idesc(AT_BN, false);
     constexpr uint32_t IDESC_O = at_idesc(DH, true);
     const uint32_t tO = tmem + 256;
-    bool ok = at_wait_warp(&q_full, 0, abort_flag, p.err, wlim);
-    tc_fence_after();
-    auto issue_s = [&](int it) {
+    bool ok = true;
+    const int total = nit * nh;
+    auto issue_s = [&](int it, int hb, bool last) {   // hb: the head's Q buffer; last: its last key tile
       const int s = it & 1;
       tc_fence_after();
       if (elect_one()) {
         const uint32_t d = tmem + (uint32_t)(s * 128);
 #pragma unroll
         for (int kk = 0; kk < DH / 16; ++kk) {
-          const uint64_t a = sdesc_sw128(smem_u32(sQ + (kk >> 2) * AT_BM * 128) + (kk & 3) * 32);
+          const uint64_t a = sdesc_sw128(smem_u32(sQ + hb * L::Q_BYTES + (kk >> 2) * AT_BM * 128) + (kk & 3) * 32);
           const uint64_t b = sdesc_sw128(smem_u32(sK + s * L::KV_BYTES + (kk >> 2) * AT_BN * 128) + (kk & 3) * 32);
           umma_bf16(d, a, b, IDESC_S, kk > 0 ? 1u : 0u);
         }
         umma_commit(&s_full[s]);
         umma_commit(&k_empty[s]);
+        if (last) umma_commit(&q_free[hb]);
       }
       __syncwarp();
     };
     int ns = 0, npv = 0;   // next S and next O (P V) to issue
-    int g = 0, j = 0;      // run and key tile of O npv
+    int hs = 0, js = 0;    // head and key tile within it of S ns
+    int hp = 0, jp = 0;    // of O npv
+    int g = z, j = 0;      // run and key tile of the run of O npv
     long long idle0 = clock64();
-    while (ok && npv < nit) {
+    while (ok && npv < total) {
       bool progress = false;
-      if (ns < nit) {
+      if (ns < total) {
         const int s = ns & 1;
-        bool ready = mbar_test(&k_full[s], (uint32_t)((ns >> 1) & 1)) &&
+        bool ready = (js > 0 || mbar_test(&q_full[hs % QB], (uint32_t)((hs / QB) & 1))) &&
+                     mbar_test(&k_full[s], (uint32_t)((ns >> 1) & 1)) &&
                      (ns < 2 || mbar_test(&s_free[s], (uint32_t)(((ns >> 1) - 1) & 1)));
         ready = __shfl_sync(0xffffffffu, ready ? 1 : 0, 0) != 0;
         if (ready) {
           // every lane observes the completions before the tensor core reads the stage
+          if (js == 0) at_wait_warp(&q_full[hs % QB], (uint32_t)((hs / QB) & 1), abort_flag, p.err, wlim);
           at_wait_warp(&k_full[s], (uint32_t)((ns >> 1) & 1), abort_flag, p.err, wlim);
           if (ns >= 2) at_wait_warp(&s_free[s], (uint32_t)(((ns >> 1) - 1) & 1), abort_flag, p.err, wlim);
-          issue_s(ns);
+          issue_s(ns, hs % QB, js == nit - 1);
           ++ns;
+          if (++js == nit) {
+            js = 0;
+            ++hs;
+          }
           progress = true;
         }
       }
       if (npv < ns) {
         const int s = npv & 1;
-        bool ready = mbar_test(&p_full[s], (uint32_t)((npv >> 1) & 1)) &&
+        // (the head's O buffer is free once O of the head before the previous one is out)
+        const bool o_wait = jp == 0 && hp >= QB;
+        bool ready = (!o_wait || mbar_test(&o_free[hp % QB], (uint32_t)((hp / QB - 1) & 1))) &&
+                     mbar_test(&p_full[s], (uint32_t)((npv >> 1) & 1)) &&
                      mbar_test(&v_full[s], (uint32_t)((npv >> 1) & 1));
         ready = __shfl_sync(0xffffffffu, ready ? 1 : 0, 0) != 0;
         if (ready) {
+          if (o_wait) at_wait_warp(&o_free[hp % QB], (uint32_t)((hp / QB - 1) & 1), abort_flag, p.err, wlim);
           at_wait_warp(&p_full[s], (uint32_t)((npv >> 1) & 1), abort_flag, p.err, wlim);
           at_wait_warp(&v_full[s], (uint32_t)((npv >> 1) & 1), abort_flag, p.err, wlim);
           const int nvalid = s_seg_kend[g] - j * AT_BN;
@@ -403,7 +456,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
 #pragma unroll
             for (int kk = 0; kk < AT_BN / 16; ++kk) {
               const uint64_t b = sdesc_mn_sw128(smem_u32(sV + s * L::KV_BYTES + kk * 16 * 128), (uint32_t)(AT_BN * 128));
-              umma_bf16_ts(tO, pa + (uint32_t)(kk * 8), b, IDESC_O, (npv > 0 || kk > 0) ? 1u : 0u);
+              umma_bf16_ts(tO + (uint32_t)(hp % QB * DH), pa + (uint32_t)(kk * 8), b, IDESC_O, (jp > 0 || kk > 0) ? 1u : 0u);
             }
             umma_commit(&pv_done[npv & 1]);
             umma_commit(&v_empty[s]);
@@ -411,9 +464,14 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
           __syncwarp();
           if (++j == (s_seg_kend[g] + AT_BN - 1) / AT_BN) {
             j = 0;
-            ++g;
+            g += Z;
           }
           ++npv;
+          if (++jp == nit) {
+            jp = 0;
+            ++hp;
+            g = z;
+          }
           progress = true;
         }
       }
@@ -448,120 +506,144 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
     const int t = q4 * 32 + lane;
     const uint32_t lane_base = (uint32_t)(q4 * 32) << 16;
     const int rsq = s_rseq[t], rpos = s_rpos[t];
-    float m = -INFINITY, l = 0.f;
+    const bool mine = rsq >= 0 && s_rrun[t] % Z == z;   // this CTA's row
     bool ok = true;
-    int it = 0;
+    int it = 0, kx = 0;   // key tiles, exchanges so far
     constexpr int OC = DH / 64;   // 32-column chunks of O per thread
-    auto pair_exchange = [&](float mine, int k) -> float {   // value of the partner thread
-      s_xch[k & 1][half][t] = mine;
+    auto pair_exchange = [&](float own) -> float {   // value of the partner thread
+      const int k = kx++;
+      s_xch[k & 1][half][t] = own;
       __syncwarp();
       if (lane == 0) mbar_arrive(&pair_bar[q4]);
-      if (!(ok = at_wait_warp(&pair_bar[q4], (uint32_t)(k & 1), abort_flag, p.err, wlim))) return mine;
+      if (!(ok = at_wait_warp(&pair_bar[q4], (uint32_t)(k & 1), abort_flag, p.err, wlim))) return own;
       return s_xch[k & 1][half ^ 1][t];
     };
-    for (int g = 0; g < nseg && ok; ++g) {
-      const int sq = s_seg_sq[g], kend = s_seg_kend[g];
-      const bool in_seg = rsq == sq;
-      const int kend_r = in_seg ? (p.causal ? rpos + 1 : kend) : 0;
-      const int nt = (kend + AT_BN - 1) / AT_BN;
-      for (int j = 0; j < nt; ++j, ++it) {
-        const int b = it & 1;
-        if (!(ok = at_wait_warp(&s_full[b], (uint32_t)((it >> 1) & 1), abort_flag, p.err, wlim))) break;
-        tc_fence_after();
-        // two passes over this thread's 64 S columns: the maximum, then exp2, the sum and the
-        // bf16 P; 8 partial chains
-        const int nk = min(max(kend_r - j * AT_BN, 0), AT_BN);
-        const uint32_t s_addr = tmem + lane_base + (uint32_t)(b * 128);
-        const float sc = p.scale_log2;
-        float mx[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) mx[q] = -INFINITY;
-        // this thread's 64 columns in one load, kept in registers for both passes
-        float sv[64];
-        tmem_ld64(s_addr + (uint32_t)(half * 64), sv);
-        const int k0 = half * 64;
-#pragma unroll
-        for (int e = 0; e < 64; ++e) {
-          sv[e] = k0 + e < nk ? sv[e] * sc : -INFINITY;
-          mx[e & 7] = fmaxf(mx[e & 7], sv[e]);
-        }
-        float tmax = fmaxf(fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])),
-                           fmaxf(fmaxf(mx[4], mx[5]), fmaxf(mx[6], mx[7])));
-        tmax = fmaxf(tmax, pair_exchange(tmax, it));
-        if (!ok) break;
-        float m_new = m;
-        if (tmax > m && (m == -INFINITY || tmax - m > AT_RESCALE_LOG2)) m_new = tmax;
-        const float factor = (m == -INFINITY || m_new == m) ? 1.f : exp2f(m - m_new);
-        // masked keys take exp2(-inf) = 0; a row with no key here keeps m = -inf and takes 0
-        const float mref = m_new == -INFINITY ? 0.f : m_new;
-        // P's buffer (two in TMEM) is free once O of the tile before the previous one is done;
-        // a rescale of O also needs O of the previous tile
-        if (it >= 2 && !(ok = at_wait_warp(&pv_done[it & 1], (uint32_t)(((it >> 1) - 1) & 1), abort_flag, p.err, wlim)))
-          break;
-        const bool rescale = __any_sync(0xffffffffu, factor != 1.f) != 0;
-        if (rescale && it >= 1 &&
-            !(ok = at_wait_warp(&pv_done[(it - 1) & 1], (uint32_t)(((it - 1) >> 1) & 1), abort_flag, p.err, wlim)))
-          break;
-        tc_fence_after();
-        if (rescale) {
+    // O / l of the head whose key tiles are through (the last of them done_it) to the output: in the next head only after
+    // its first P, so that the wait for O overlaps it
+    int done_h = -1, done_it = 0;
+    float done_l = 0.f;
+    auto finish = [&]() {
+      const int hh = done_h;
+      float l = done_l;
+      done_h = -1;
+      if (ok && nit > 0)
+        ok = at_wait_warp(&pv_done[done_it & 1], (uint32_t)((done_it >> 1) & 1), abort_flag, p.err, wlim);
+      if (ok) l += pair_exchange(l);
+      tc_fence_after();
+      const float inv = l > 0.f ? 1.f / l : 0.f;
 #pragma unroll 1
-          for (int c = half * OC; c < half * OC + OC; ++c) {
-            float v[32];
-            tmem_ld32(tmem + lane_base + (uint32_t)(256 + c * 32), v);
+      for (int c = half * OC; c < half * OC + OC; ++c) {
+        float v[32];
+        tmem_ld32(tmem + lane_base + (uint32_t)(256 + hh % QB * DH + c * 32), v);
+        if (ok && mine) {
+          uint32_t w[16];
 #pragma unroll
-            for (int e = 0; e < 32; ++e) v[e] *= factor;
-            tmem_st32(tmem + lane_base + (uint32_t)(256 + c * 32), v);
+          for (int e = 0; e < 16; ++e) {
+            const __nv_bfloat162 pr = __floats2bfloat162_rn(v[2 * e] * inv, v[2 * e + 1] * inv);
+            w[e] = *reinterpret_cast<const uint32_t*>(&pr);
           }
-          tmem_st_wait();
-        }
-        float sm[8];
+          uint4* o = reinterpret_cast<uint4*>(p.out + (size_t)(r0 + t) * p.ld_out + (h0 + hh) * DH + c * 32);
 #pragma unroll
-        for (int q = 0; q < 8; ++q) sm[q] = 0.f;
-        uint32_t pk[32];
-#pragma unroll
-        for (int e = 0; e < 64; e += 2) {
-          const float p0 = ex2_approx(sv[e] - mref);   // masked keys: exp2(-inf) = 0
-          const float p1 = ex2_approx(sv[e + 1] - mref);
-          sm[(e >> 1) & 7] += p0 + p1;
-          const __nv_bfloat162 pr = __floats2bfloat162_rn(p0, p1);
-          pk[e >> 1] = *reinterpret_cast<const uint32_t*>(&pr);
+          for (int e = 0; e < 4; ++e) o[e] = make_uint4(w[4 * e], w[4 * e + 1], w[4 * e + 2], w[4 * e + 3]);
         }
-        // this thread's keys -> P columns half*32 .. +31 of this tile's buffer (2 keys a column)
-        tmem_st32u(tmem + lane_base + (uint32_t)(384 + (it & 1) * 64 + half * 32), pk);
-        tmem_st_wait();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&s_free[b]);   // S of this buffer is read
-        const float rs = ((sm[0] + sm[1]) + (sm[2] + sm[3])) + ((sm[4] + sm[5]) + (sm[6] + sm[7]));
-        l = l * factor + rs;   // this thread's keys; the pair's sums are added at the end
-        m = m_new;
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&p_full[it & 1]);
       }
-    }
-    if (ok && nit > 0)
-      ok = at_wait_warp(&pv_done[(nit - 1) & 1], (uint32_t)(((nit - 1) >> 1) & 1), abort_flag, p.err, wlim);
-    if (ok) l += pair_exchange(l, it);
-    tc_fence_after();
-    const int r = r0 + t;
-    const float inv = l > 0.f ? 1.f / l : 0.f;
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&o_free[hh % QB]);   // the head's O is read
+    };
+    for (int hh = 0; hh < nh && ok; ++hh) {
+      float m = -INFINITY, l = 0.f;
+      const uint32_t o_col = 256u + (uint32_t)(hh % QB * DH);   // the head's O
+      for (int g = z; g < nseg && ok; g += Z) {
+        const int sq = s_seg_sq[g], kend = s_seg_kend[g];
+        const bool in_seg = rsq == sq;
+        const int kend_r = in_seg ? (p.causal ? rpos + 1 : kend) : 0;
+        const int nt = (kend + AT_BN - 1) / AT_BN;
+        for (int j = 0; j < nt; ++j, ++it) {
+          const int b = it & 1;
+          if (!(ok = at_wait_warp(&s_full[b], (uint32_t)((it >> 1) & 1), abort_flag, p.err, wlim))) break;
+          tc_fence_after();
+          // two passes over this thread's 64 S columns: the maximum, then exp2, the sum and the
+          // bf16 P; 8 partial chains
+          const int nk = min(max(kend_r - j * AT_BN, 0), AT_BN);
+          const uint32_t s_addr = tmem + lane_base + (uint32_t)(b * 128);
+          const float sc = p.scale_log2;
+          float mx[8];
+#pragma unroll
+          for (int q = 0; q < 8; ++q) mx[q] = -INFINITY;
+          // this thread's 64 columns in one load, kept in registers for both passes
+          float sv[64];
+          tmem_ld64(s_addr + (uint32_t)(half * 64), sv);
+          const int k0 = half * 64;
+#pragma unroll
+          for (int e = 0; e < 64; ++e) {
+            sv[e] = k0 + e < nk ? sv[e] * sc : -INFINITY;
+            mx[e & 7] = fmaxf(mx[e & 7], sv[e]);
+          }
+          float tmax = fmaxf(fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])),
+                             fmaxf(fmaxf(mx[4], mx[5]), fmaxf(mx[6], mx[7])));
+          tmax = fmaxf(tmax, pair_exchange(tmax));
+          if (!ok) break;
+          float m_new = m;
+          if (tmax > m && (m == -INFINITY || tmax - m > AT_RESCALE_LOG2)) m_new = tmax;
+          const float factor = (m == -INFINITY || m_new == m) ? 1.f : exp2f(m - m_new);
+          // masked keys take exp2(-inf) = 0; a row with no key here keeps m = -inf and takes 0
+          const float mref = m_new == -INFINITY ? 0.f : m_new;
+          // P's buffer (two in TMEM) is free once O of the tile before the previous one is done;
+          // a rescale of O also needs O of the previous tile
+          if (it >= 2 && !(ok = at_wait_warp(&pv_done[it & 1], (uint32_t)(((it >> 1) - 1) & 1), abort_flag, p.err, wlim)))
+            break;
+          const bool rescale = __any_sync(0xffffffffu, factor != 1.f) != 0;
+          if (rescale && it >= 1 &&
+              !(ok = at_wait_warp(&pv_done[(it - 1) & 1], (uint32_t)(((it - 1) >> 1) & 1), abort_flag, p.err, wlim)))
+            break;
+          tc_fence_after();
+          if (rescale) {
 #pragma unroll 1
-    for (int c = half * OC; c < half * OC + OC; ++c) {
-      float v[32];
-      tmem_ld32(tmem + lane_base + (uint32_t)(256 + c * 32), v);
-      if (ok && rsq >= 0) {
-        uint32_t w[16];
+            for (int c = half * OC; c < half * OC + OC; ++c) {
+              float v[32];
+              tmem_ld32(tmem + lane_base + o_col + (uint32_t)(c * 32), v);
 #pragma unroll
-        for (int e = 0; e < 16; ++e) {
-          const __nv_bfloat162 pr = __floats2bfloat162_rn(v[2 * e] * inv, v[2 * e + 1] * inv);
-          w[e] = *reinterpret_cast<const uint32_t*>(&pr);
+              for (int e = 0; e < 32; ++e) v[e] *= factor;
+              tmem_st32(tmem + lane_base + o_col + (uint32_t)(c * 32), v);
+            }
+            tmem_st_wait();
+          }
+          float sm[8];
+#pragma unroll
+          for (int q = 0; q < 8; ++q) sm[q] = 0.f;
+          uint32_t pk[32];
+#pragma unroll
+          for (int e = 0; e < 64; e += 2) {
+            const float p0 = ex2_approx(sv[e] - mref);   // masked keys: exp2(-inf) = 0
+            const float p1 = ex2_approx(sv[e + 1] - mref);
+            sm[(e >> 1) & 7] += p0 + p1;
+            const __nv_bfloat162 pr = __floats2bfloat162_rn(p0, p1);
+            pk[e >> 1] = *reinterpret_cast<const uint32_t*>(&pr);
+          }
+          // this thread's keys -> P columns half*32 .. +31 of this tile's buffer (2 keys a column)
+          tmem_st32u(tmem + lane_base + (uint32_t)(384 + (it & 1) * 64 + half * 32), pk);
+          tmem_st_wait();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&s_free[b]);   // S of this buffer is read
+          const float rs = ((sm[0] + sm[1]) + (sm[2] + sm[3])) + ((sm[4] + sm[5]) + (sm[6] + sm[7]));
+          l = l * factor + rs;   // this thread's keys; the pair's sums are added at the end
+          m = m_new;
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&p_full[it & 1]);
+          if (QB > 1 && done_h >= 0) {
+            finish();
+            if (!ok) break;
+          }
         }
-        uint4* o = reinterpret_cast<uint4*>(p.out + (size_t)r * p.ld_out + h * DH + c * 32);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) o[e] = make_uint4(w[4 * e], w[4 * e + 1], w[4 * e + 2], w[4 * e + 3]);
       }
+      done_h = hh;
+      done_it = it - 1;
+      done_l = l;
     }
+    if (done_h >= 0) finish();
   }
   tc_fence_before();
   __syncthreads();
@@ -576,7 +658,7 @@ bool g_at_attr[2] = {false, false};
 int launch_attention_tc(cudaStream_t st, const void* q, int ld_q, int q_rows, void* out, int ld_out, DevRange rows,
                         int max_rows, const int* row_tok, const int* tok_seq, const int* tok_pos, const int* seq_len,
                         const KVCacheView& cache, int n_layers, int layer0, int n_heads, int causal, float scale_log2,
-                        unsigned* err) {
+                        int seq_rows, unsigned* err) {
   const int dh = cache.head_dim;
   if (!tc_gemm_supported() || (dh != 64 && dh != 128) || cache.block_tokens != 16 || rows.begin) return -1;
   if (n_heads % cache.n_kv_heads || ld_q % 8 || ld_out % 8 || ((uintptr_t)q & 15) || ((uintptr_t)out & 15)) return -1;
@@ -604,7 +686,17 @@ int launch_attention_tc(cudaStream_t st, const void* q, int ld_q, int q_rows, vo
   prm.causal = causal;
   prm.scale_log2 = scale_log2;
   prm.err = err;
-  const dim3 grid((max_rows + AT_BM - 1) / AT_BM, n_heads);
+  static const int sms = [] {
+    int dev = 0, n = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    return std::max(1, n);
+  }();
+  // short sequences in few tiles: as many CTAs per (tile, head) as sequences in a tile and idle SMs allow
+  const int tiles = (max_rows + AT_BM - 1) / AT_BM;
+  prm.sms = sms;
+  prm.z = std::max(1, std::min({AT_MAX_Z, sms / (tiles * n_heads), seq_rows > 0 ? AT_BM / seq_rows : 1}));
+  const dim3 grid(tiles * n_heads * prm.z);
   cudaError_t e;
   if (dh == 128) {
     const size_t smem = AtLayout<128>::TOTAL + 1024;

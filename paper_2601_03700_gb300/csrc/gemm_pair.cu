@@ -23,7 +23,7 @@
 // CTA = 10 warps: warp 0 lane 0 TMA producer; warp 1 tensor-memory allocator, its lane 0 in CTA 0 issues the pair's MMAs;
 // warps 2..9 epilogue. Ring of k-blocks with full barriers in CTA 0 (both CTAs' copies complete on it) and empty barriers in
 // both; two accumulator buffers. Waits are bounded: on time-out a CTA sets ERRW_TIMEOUT, stops, and leaves with its peer.
-#define ADEPT_TU_ID 11
+#define ADEPT_TU_ID 12
 #include "gemm_pair.h"
 #include "epilogue.cuh"
 #include "gemm_tc.h"

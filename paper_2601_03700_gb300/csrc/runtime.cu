@@ -1227,7 +1227,7 @@ static adept_status run_pass(adept_model* m, int n_tok, int batch, int prompt_le
         prof_begin(m, ADEPT_PROF_ATTENTION, st, &b);
         launch_attention(st, m->dt, m->q, Dq, m->att, Dq, act, mr, rt, m->tok_seq, m->tok_pos, m->d_src_len,
                          cross_view(m), l0, m->H, 0, decode ? m->cs_blocks_per_seq * c.kv_block_tokens : 0,
-                         m->attn_ws, m->attn_ctr, m->err_word, nullptr, 0, m->use_attn_tc ? m->T_max : 0, N);
+                         m->attn_ws, m->attn_ctr, m->err_word, nullptr, prompt_len, m->use_attn_tc ? m->T_max : 0, N);
         prof_end(m, ADEPT_PROF_ATTENTION, st, b, 0, 0);
         m->launches += 1;
       }
