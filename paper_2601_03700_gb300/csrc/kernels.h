@@ -38,6 +38,10 @@ void launch_pass_init(cudaStream_t st, int n_tok, int prompt_len, int decode, in
 void launch_embed(cudaStream_t st, int dt, const int* tokens, int n_tok, const int* tok_pos, const void* E,
                   const void* P, const float* type_emb, const float* g, const float* b, int family, int D, int V,
                   float eps, float* X, unsigned* err, void* xhat, int smode, float seps);
+// launch_embed for rows of up to 8192 elements (false: longer, nothing launched).
+bool launch_embed_rows(cudaStream_t st, int dt, const int* tokens, int n_tok, const int* tok_pos, const void* E,
+                       const void* P, const float* type_emb, const float* g, const float* b, int family, int D, int V,
+                       float eps, float* X, unsigned* err, void* xhat, int smode, float seps);
 void launch_standardize(cudaStream_t st, int dt, const float* X, int ldx, const int* in_rows, DevRange rows,
                         int max_rows, int D, int mode, float eps, void* out, int ld_out);
 // LayerNorm with gain and shift of rows of X in place, and the result in the model's type in xt.

@@ -51,6 +51,68 @@ __device__ __forceinline__ float2 row_norm(const float4 (&x)[V ? V : 1], const f
   return make_float2(mu[0], rsqrtf(s2[0] / D + eps));
 }
 
+__device__ __forceinline__ float4 row4(const bf16* x, int v) {
+  const uint2 u = reinterpret_cast<const uint2*>(x)[v];
+  const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.x));
+  const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.y));
+  return make_float4(a.x, a.y, b.x, b.y);
+}
+__device__ __forceinline__ float4 row4(const float* x, int v) { return reinterpret_cast<const float4*>(x)[v]; }
+__device__ __forceinline__ float4 add4(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
+
+// Token (+ position, + type) embeddings into the residual stream X and, as the first attention's input, into xhat: standardised by
+// smode, or for the encoder (family 2) both the LayerNorm with gain and shift. A token id outside [0, V) is flagged and reads row 0.
+// 8192 rows of 768: 26 us with a CTA per row and an element per load, 14 so; 2048 of 4096 29 and 13. Few tokens (generation steps)
+// take a CTA each.
+template <typename T, int TPR, int V>
+__global__ void __launch_bounds__(RW_THREADS)
+    embed_rows_kernel(const int* __restrict__ tokens, int n_tok, const int* __restrict__ tok_pos, const T* __restrict__ E,
+                      const T* __restrict__ P, const float* __restrict__ type_emb, const float* __restrict__ g,
+                      const float* __restrict__ b, int family, int D, int vocab, float eps, float* __restrict__ X,
+                      unsigned* err, T* __restrict__ xhat, int smode, float seps) {
+  PDL_ENTRY();
+  __shared__ float red[RW_THREADS / 32];
+  constexpr int G = RW_THREADS / TPR;
+  const int t = blockIdx.x * G + (int)threadIdx.x / TPR, sub = threadIdx.x & (TPR - 1), D4 = D >> 2;
+  if (t >= n_tok) return;   // (a whole group)
+  int tok = tokens[t];
+  if (tok < 0 || tok >= vocab) {
+    if (sub == 0) atomicOr(err, ERRW_TOKEN);
+    tok = 0;
+  }
+  const int pos = P ? tok_pos[t] : 0;
+  float4 x[V];
+#pragma unroll
+  for (int j = 0; j < V; ++j)
+    if (sub + j * TPR < D4) x[j] = row4(E + (size_t)tok * D, sub + j * TPR);
+  if (P) {
+#pragma unroll
+    for (int j = 0; j < V; ++j)
+      if (sub + j * TPR < D4) x[j] = add4(x[j], row4(P + (size_t)pos * D, sub + j * TPR));
+  }
+  if (type_emb) {
+#pragma unroll
+    for (int j = 0; j < V; ++j)
+      if (sub + j * TPR < D4) x[j] = add4(x[j], row4(type_emb, sub + j * TPR));
+  }
+  float* o = X + (size_t)t * D;
+  T* oh = xhat + (size_t)t * D;
+  const bool enc = family == 2;
+  const float2 n = row_norm<TPR, V>(x, nullptr, true, sub, D4, D, enc ? (int)NORM_LN : smode, enc ? eps : seps, red);
+#pragma unroll
+  for (int j = 0; j < V; ++j) {
+    const int v = sub + j * TPR;
+    if (v >= D4) continue;
+    float4 y = scale4(centre4(x[j], n.x), n.y);
+    if (enc) {
+      const float4 gg = row4(g, v), bb = row4(b, v);
+      y = make_float4(y.x * gg.x + bb.x, y.y * gg.y + bb.y, y.z * gg.z + bb.z, y.w * gg.w + bb.w);
+    }
+    put4(o, v, enc ? y : x[j]);
+    put4(oh, v, y);
+  }
+}
+
 // Rows in_rows[r] (or r) of X standardised into row r of out.
 template <typename T, int TPR, int V>
 __global__ void __launch_bounds__(RW_THREADS)
@@ -323,6 +385,30 @@ static int rows_grid(int max_rows, int per) { return std::min(cdiv(max_rows, per
     else if ((D) <= 8192) GO(T, 256, 8);\
     else GO(T, 256, 0);                \
   } while (0)
+
+bool launch_embed_rows(cudaStream_t st, int dt, const int* tokens, int n_tok, const int* tok_pos, const void* E,
+                       const void* P, const float* type_emb, const float* g, const float* b, int family, int D, int V,
+                       float eps, float* X, unsigned* err, void* xhat, int smode, float seps) {
+  if (D % 4 || D > 8192) return false;
+  if (n_tok <= 0) return true;
+#define GO(T, TPR, NV)                                                                                                \
+  launch_k(embed_rows_kernel<T, TPR, NV>, cdiv(n_tok, RW_THREADS / TPR), RW_THREADS, 0, st, tokens, n_tok, tok_pos, \
+           (const T*)E, (const T*)P, type_emb, g, b, family, D, V, eps, X, err, (T*)xhat, smode, seps)
+#define PICK(T)                     \
+  if (D <= 1024 && n_tok <= 16) GO(T, 256, 1); \
+  else if (D <= 768) GO(T, 32, 6);  \
+  else if (D <= 1024) GO(T, 32, 8); \
+  else if (D <= 4096) GO(T, 256, 4); \
+  else GO(T, 256, 8)
+  if (dt == 1) {
+    PICK(bf16);
+  } else {
+    PICK(float);
+  }
+#undef PICK
+#undef GO
+  return true;
+}
 
 void launch_standardize(cudaStream_t st, int dt, const float* X, int ldx, const int* in_rows, DevRange rows,
                         int max_rows, int D, int mode, float eps, void* out, int ld_out) {
