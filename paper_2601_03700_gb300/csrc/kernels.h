@@ -30,9 +30,9 @@ static __device__ __forceinline__ float exit_similarity(int metric, float ns, fl
 // Token -> (sequence, position) maps, identity row map, the pass's counters (all rows
 // active), if sim is given NaN for every (token, layer) similarity, and if tok_exit is
 // given N as every token's exit layer so far.
-void launch_pass_init(cudaStream_t st, int n_tok, int prompt_len, int decode, int* tok_seq, int* tok_pos,
-                      int* row_tok, int* seq_len, int seq_cap, int max_pos, unsigned* err, int* ctr, int n_ctr,
-                      float* sim, int n_layers, int* tok_exit);
+void launch_pass_init(cudaStream_t st, int n_tok, int prompt_len, int* tok_seq, int* tok_pos, int* row_tok, int* seq_len,
+                      int seq_cap, int max_pos, unsigned* err, int* ctr, int n_ctr, float* sim, int n_layers,
+                      int* tok_exit);
 // xhat: the embedded rows as the first layer's attention input (decoders: standardised by smode,
 // seps) in the model's type, [n_tok][D].
 void launch_embed(cudaStream_t st, int dt, const int* tokens, int n_tok, const int* tok_pos, const void* E,
@@ -69,13 +69,15 @@ void launch_exit_rows(cudaStream_t st, int dt, const float* Xin, const float* Xo
                       const int* tok_pos, unsigned* err);
 void launch_set_float(cudaStream_t st, float* p, float v);
 void launch_span_collect(cudaStream_t st, SpanSite* sites, int n, SpanTotal* tot, int n_cls);
-// Generation-step staging of the caller's inputs (forced NULL -> zeros) and outputs (each
-// output optional).
-void launch_stage_in(cudaStream_t st, float* d_delta, float delta, const int* tokens, int* dec_tok, const int* forced,
-                     int* dec_forced, int batch);
-void launch_stage_out(cudaStream_t st, int batch, const int* dec_exit, int* exit_out, const int* dec_next,
-                      int* next_out, const float* logits, float* logits_out, long long n_logits, const float* sim,
-                      float* sim_out, int n_sim);
+// Generation-step staging of the caller's inputs (forced NULL -> zeros) with the pass's set-up, and of the
+// outputs (each optional) with the greedy tokens.
+void launch_step_in(cudaStream_t st, float* d_delta, float delta, const int* tokens, int* dec_tok, const int* forced,
+                    int* dec_forced, int batch, int* tok_seq, int* tok_pos, int* row_tok, int* seq_len, int seq_cap,
+                    int max_pos, unsigned* err, int* ctr, int n_ctr, float* sim, int n_layers);
+// part_v / part_i: 32 per row; cnt: one per row, 0 before and after.
+void launch_step_out(cudaStream_t st, int batch, int V, const float* logits, float* logits_out, int* next_out, float* part_v,
+                     int* part_i, unsigned* cnt, const int* dec_exit, int* exit_out, const float* sim, float* sim_out,
+                     int n_sim);
 void launch_final_scatter(cudaStream_t st, const float* X, int D, const int* n_rows, int max_rows, const int* row_tok,
                           float* final_, int* exit_layer_out, int n_layers);
 // launch_final_scatter that also writes each row standardised for the output head (hmode, heps)

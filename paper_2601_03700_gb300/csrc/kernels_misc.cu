@@ -13,11 +13,10 @@ namespace adept {
 // ---------------------------------------------------------------------------
 // pass set-up: token -> (sequence, position), identity row map, counters
 // ---------------------------------------------------------------------------
-__global__ void pass_init_kernel(int n_tok, int prompt_len, int decode, int* tok_seq, int* tok_pos,
-                                 int* row_tok, int* seq_len, int seq_cap, int max_pos, unsigned* err, int* ctr,
-                                 int n_ctr, float* sim, int n_layers, int* tok_exit) {
-  PDL_ENTRY();
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+// Thread t's part: counter t, token t.
+__device__ __forceinline__ void pass_init(int t, int n_tok, int prompt_len, int decode, int* tok_seq, int* tok_pos,
+                                          int* row_tok, int* seq_len, int seq_cap, int max_pos, unsigned* err, int* ctr,
+                                          int n_ctr, float* sim, int n_layers, int* tok_exit) {
   // the pass's counters: all active, nothing exited
   if (t < n_ctr) ctr[t] = t == CTR_ACTIVE ? n_tok : 0;
   if (t >= n_tok) return;
@@ -43,6 +42,13 @@ __global__ void pass_init_kernel(int n_tok, int prompt_len, int decode, int* tok
   tok_seq[t] = s;
   tok_pos[t] = p;
   row_tok[t] = t;
+}
+__global__ void pass_init_kernel(int n_tok, int prompt_len, int* tok_seq, int* tok_pos, int* row_tok, int* seq_len,
+                                 int seq_cap, int max_pos, unsigned* err, int* ctr, int n_ctr, float* sim, int n_layers,
+                                 int* tok_exit) {
+  PDL_ENTRY();
+  pass_init(blockIdx.x * blockDim.x + threadIdx.x, n_tok, prompt_len, 0, tok_seq, tok_pos, row_tok, seq_len, seq_cap,
+            max_pos, err, ctr, n_ctr, sim, n_layers, tok_exit);
 }
 
 // ---------------------------------------------------------------------------
@@ -381,43 +387,25 @@ void launch_span_collect(cudaStream_t st, SpanSite* sites, int n, SpanTotal* tot
   launch_k(span_collect_kernel, 1, 1024, 0, st, sites, n, tot, n_cls);
 }
 
-// Generation-step staging: the caller's inputs into the library's fixed buffers (the captured
-// step reads only those), in one launch instead of a kernel and two copies.
-__global__ void stage_in_kernel(float* d_delta, float delta, const int* tokens, int* dec_tok, const int* forced,
-                                int* dec_forced, int batch) {
+// The start of a generation step: the caller's inputs into the library's fixed buffers (the captured step reads only those)
+// and the pass's set-up, in one launch before the captured step (a set-up of its own within it took 2.2 us).
+__global__ void step_in_kernel(float* d_delta, float delta, const int* tokens, int* dec_tok, const int* forced,
+                               int* dec_forced, int batch, int* tok_seq, int* tok_pos, int* row_tok, int* seq_len,
+                               int seq_cap, int max_pos, unsigned* err, int* ctr, int n_ctr, float* sim, int n_layers) {
   PDL_ENTRY();
-  if (threadIdx.x == 0) *d_delta = delta;
-  for (int b = threadIdx.x; b < batch; b += blockDim.x) {
-    dec_tok[b] = tokens[b];
-    dec_forced[b] = forced ? forced[b] : 0;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t == 0) *d_delta = delta;
+  if (t < batch) {
+    dec_tok[t] = tokens[t];
+    dec_forced[t] = forced ? forced[t] : 0;
   }
+  pass_init(t, batch, 1, 1, tok_seq, tok_pos, row_tok, seq_len, seq_cap, max_pos, err, ctr, n_ctr, sim, n_layers, nullptr);
 }
-void launch_stage_in(cudaStream_t st, float* d_delta, float delta, const int* tokens, int* dec_tok, const int* forced,
-                     int* dec_forced, int batch) {
-  launch_k(stage_in_kernel, 1, 32, 0, st, d_delta, delta, tokens, dec_tok, forced, dec_forced, batch);
-}
-
-// ... and the step's outputs out of them into the caller's buffers (each optional).
-__global__ void stage_out_kernel(int batch, const int* dec_exit, int* exit_out, const int* dec_next, int* next_out,
-                                 const float* logits, float* logits_out, long long n_logits, const float* sim,
-                                 float* sim_out, int n_sim) {
-  PDL_ENTRY();
-  const long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
-  for (long long i = i0; i < batch; i += step) {
-    if (exit_out) exit_out[i] = dec_exit[i];
-    if (next_out) next_out[i] = dec_next[i];
-  }
-  if (sim_out)
-    for (long long i = i0; i < n_sim; i += step) sim_out[i] = sim[i];
-  if (logits_out)
-    for (long long i = i0; i < n_logits; i += step) logits_out[i] = logits[i];
-}
-void launch_stage_out(cudaStream_t st, int batch, const int* dec_exit, int* exit_out, const int* dec_next,
-                      int* next_out, const float* logits, float* logits_out, long long n_logits, const float* sim,
-                      float* sim_out, int n_sim) {
-  const int grid = logits_out ? (int)std::min<long long>(304, (n_logits + 255) / 256) : 1;
-  launch_k(stage_out_kernel, std::max(grid, 1), 256, 0, st, batch, dec_exit, exit_out, dec_next, next_out, logits,
-           logits_out, n_logits, sim, sim_out, n_sim);
+void launch_step_in(cudaStream_t st, float* d_delta, float delta, const int* tokens, int* dec_tok, const int* forced,
+                    int* dec_forced, int batch, int* tok_seq, int* tok_pos, int* row_tok, int* seq_len, int seq_cap,
+                    int max_pos, unsigned* err, int* ctr, int n_ctr, float* sim, int n_layers) {
+  launch_k(step_in_kernel, cdiv(std::max(batch, n_ctr), 256), 256, 0, st, d_delta, delta, tokens, dec_tok, forced,
+           dec_forced, batch, tok_seq, tok_pos, row_tok, seq_len, seq_cap, max_pos, err, ctr, n_ctr, sim, n_layers);
 }
 
 // After layer N: the remaining active rows' s_N are their final states.
@@ -1039,10 +1027,10 @@ __global__ void __launch_bounds__(256) read_kv_kernel(KVCacheView c, int row_byt
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
-void launch_pass_init(cudaStream_t st, int n_tok, int prompt_len, int decode, int* tok_seq, int* tok_pos,
-                      int* row_tok, int* seq_len, int seq_cap, int max_pos, unsigned* err, int* ctr, int n_ctr,
-                      float* sim, int n_layers, int* tok_exit) {
-  launch_k(pass_init_kernel, cdiv(std::max(n_tok, n_ctr), 256), 256, 0, st, n_tok, prompt_len, decode, tok_seq, tok_pos,
+void launch_pass_init(cudaStream_t st, int n_tok, int prompt_len, int* tok_seq, int* tok_pos, int* row_tok, int* seq_len,
+                      int seq_cap, int max_pos, unsigned* err, int* ctr, int n_ctr, float* sim, int n_layers,
+                      int* tok_exit) {
+  launch_k(pass_init_kernel, cdiv(std::max(n_tok, n_ctr), 256), 256, 0, st, n_tok, prompt_len, tok_seq, tok_pos,
            row_tok, seq_len, seq_cap, max_pos, err, ctr, n_ctr, sim, n_layers, tok_exit);
 }
 
@@ -1244,6 +1232,104 @@ __global__ void argmax_merge_kernel(const float* pv, const int* pi, int rows, in
     }
   }
   out[r] = bi == 0x7fffffff ? 0 : bi;
+}
+
+// The end of a generation step: its outputs out of the library's buffers into the caller's (each optional), and the greedy
+// token of each row (lowest index on ties) from the logits as they pass: a CTA per row and part of the vocabulary, the last of
+// a row to arrive (cnt, left at 0) merges the parts. Argmax in two launches within the captured step and a copy after it took
+// 3.0 + 1.5 + 3.8 us at one row of 50257.
+__global__ void __launch_bounds__(256)
+    step_out_kernel(int batch, int V, int parts, const float* __restrict__ logits, float* __restrict__ logits_out,
+                    int* __restrict__ next_out, float* pv, int* pi, unsigned* cnt, const int* dec_exit, int* exit_out,
+                    const float* sim, float* sim_out, int n_sim) {
+  PDL_ENTRY();
+  const int part = blockIdx.x % parts, r = blockIdx.x / parts, tid = threadIdx.x;
+  if (part == 0 && tid == 0 && exit_out) exit_out[r] = dec_exit[r];
+  if (part == 0 && sim_out) {   // this row's similarities
+    const int n = n_sim / batch;
+    for (int i = tid; i < n; i += 256) sim_out[(size_t)r * n + i] = sim[(size_t)r * n + i];
+  }
+  if (!logits_out && !next_out) return;
+  const int chunk = (V + parts - 1) / parts, lo = part * chunk, hi = min(V, lo + chunk);
+  const float* l = logits + (size_t)r * V;
+  float* o = logits_out ? logits_out + (size_t)r * V : nullptr;
+  float bv = -INFINITY;
+  int bi = 0x7fffffff;
+  auto better = [](float v, int i, float w, int j) { return v > w || (v == w && i < j); };
+  for (int v0 = lo + tid; v0 < hi; v0 += 8 * 256) {   // 8 loads in flight
+    float x[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) x[u] = v0 + u * 256 < hi ? l[v0 + u * 256] : -INFINITY;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int v = v0 + u * 256;
+      if (v >= hi) continue;
+      if (o) o[v] = x[u];
+      if (better(x[u], v, bv, bi)) {
+        bv = x[u];
+        bi = v;
+      }
+    }
+  }
+  if (!next_out) return;
+  __shared__ float sv[8];
+  __shared__ int si[8];
+  __shared__ unsigned s_seen;
+  auto warp_best = [&]() {
+#pragma unroll
+    for (int s = 16; s; s >>= 1) {
+      const float ov = __shfl_xor_sync(0xffffffffu, bv, s);
+      const int oi = __shfl_xor_sync(0xffffffffu, bi, s);
+      if (better(ov, oi, bv, bi)) {
+        bv = ov;
+        bi = oi;
+      }
+    }
+  };
+  warp_best();
+  if ((tid & 31) == 0) {
+    sv[tid >> 5] = bv;
+    si[tid >> 5] = bi;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    for (int k = 1; k < 8; ++k)
+      if (better(sv[k], si[k], bv, bi)) {
+        bv = sv[k];
+        bi = si[k];
+      }
+    if (parts > 1) {
+      pv[r * parts + part] = bv;
+      pi[r * parts + part] = bi;
+      __threadfence();
+      s_seen = atomicAdd(&cnt[r], 1u);
+      __threadfence();
+    }
+  }
+  if (parts > 1) {
+    __syncthreads();
+    if (s_seen != (unsigned)(parts - 1) || tid >= 32) return;
+    bv = -INFINITY;
+    bi = 0x7fffffff;
+    for (int k = tid; k < parts; k += 32) {
+      const float x = __ldcg(&pv[r * parts + k]);
+      const int i = __ldcg(&pi[r * parts + k]);
+      if (better(x, i, bv, bi)) {
+        bv = x;
+        bi = i;
+      }
+    }
+    warp_best();
+    if (tid == 0) cnt[r] = 0;
+  }
+  if (tid == 0) next_out[r] = bi == 0x7fffffff ? 0 : bi;
+}
+void launch_step_out(cudaStream_t st, int batch, int V, const float* logits, float* logits_out, int* next_out, float* part_v,
+                     int* part_i, unsigned* cnt, const int* dec_exit, int* exit_out, const float* sim, float* sim_out,
+                     int n_sim) {
+  const int parts = V <= 4096 || (!logits_out && !next_out) ? 1 : ARGMAX_SPLIT;
+  launch_k(step_out_kernel, batch * parts, 256, 0, st, batch, V, parts, logits, logits_out,
+           next_out, part_v, part_i, cnt, dec_exit, exit_out, sim, sim_out, n_sim);
 }
 
 int launch_argmax(cudaStream_t st, const float* logits, int V, int rows, int* out, float* part_v, int* part_i) {

@@ -153,6 +153,7 @@ struct adept_model {
   int ds_ctas = 0;
   float* amax_v = nullptr;       // argmax partials
   int* amax_i = nullptr;
+  unsigned* amax_cnt = nullptr;   // arrivals per row, 0 between launches
   float* scratch = nullptr;
   size_t scratch_elems = 0;
   // skipped-layer fill workspace (adept_skip_kv_fill)
@@ -161,7 +162,7 @@ struct adept_model {
   int *fill_tok = nullptr, *fill_hist = nullptr, *fill_start = nullptr, *fill_cursor = nullptr;
   // generation-step staging buffers (the captured graph reads and writes only these)
   float* d_delta = nullptr;
-  int *dec_tok = nullptr, *dec_forced = nullptr, *dec_exit = nullptr, *dec_next = nullptr;
+  int *dec_tok = nullptr, *dec_forced = nullptr, *dec_exit = nullptr;
   float* dec_sim = nullptr;
   cudaStream_t cap_stream = nullptr;
   std::vector<cudaGraphExec_t> dec_graph;   // per batch size
@@ -907,7 +908,8 @@ static adept_status alloc_runtime(adept_model* m) {
   TRY(dalloc_t(m, &m->dec_tok, c.max_batch));
   TRY(dalloc_t(m, &m->dec_forced, c.max_batch));
   TRY(dalloc_t(m, &m->dec_exit, c.max_batch));
-  TRY(dalloc_t(m, &m->dec_next, c.max_batch));
+  TRY(dalloc_t(m, &m->amax_cnt, c.max_batch));
+  CUDA_TRY(m, cudaMemset(m->amax_cnt, 0, sizeof(unsigned) * c.max_batch));
   TRY(dalloc_t(m, &m->dec_sim, (size_t)c.max_batch * m->N));
   m->dec_graph.assign(c.max_batch + 1, nullptr);
   m->dec_warm.assign(c.max_batch + 1, 0);
@@ -1085,9 +1087,12 @@ static adept_status run_pass(adept_model* m, int n_tok, int batch, int prompt_le
   const bool head_x = decode && fam != ADEPT_FAMILY_BERT && m->dt == ADEPT_DTYPE_BF16 && head_rows_supported(D);
   m->xhead_ready = head_x;
   int32_t* exit_w = stop ? m->tok_exit : exit_out;
-  launch_pass_init(st, n_tok, prompt_len, decode ? 1 : 0, m->tok_seq, m->tok_pos, m->row_tok[0], m->d_seq_len,
-                   m->max_blocks_per_seq * c.kv_block_tokens, fam == ADEPT_FAMILY_LLAMA ? 0 : c.max_pos,
-                   m->err_word, m->ctr, ctr_words(N), sim_out, N, stop ? m->tok_exit : nullptr);
+  if (!decode) {   // (a generation step's is part of its first launch)
+    launch_pass_init(st, n_tok, prompt_len, m->tok_seq, m->tok_pos, m->row_tok[0], m->d_seq_len,
+                     m->max_blocks_per_seq * c.kv_block_tokens, fam == ADEPT_FAMILY_LLAMA ? 0 : c.max_pos, m->err_word,
+                     m->ctr, ctr_words(N), sim_out, N, stop ? m->tok_exit : nullptr);
+    m->launches += 1;
+  }
   // the producer of each layer's input (the embedding, then the exit step) also writes it as the
   // attention input (standardised, in the model's type) into xn; in passes of at most DG_MAX_M
   // rows (bf16 decoders) the O projection hands the tile statistics of its output to the FFN
@@ -1096,7 +1101,7 @@ static adept_status run_pass(adept_model* m, int n_tok, int batch, int prompt_le
                       fam != ADEPT_FAMILY_BERT;
   launch_embed(st, m->dt, tokens, n_tok, m->tok_pos, m->tok_emb, m->pos_emb, m->type_emb, m->emb_g, m->emb_b, fam, D,
                m->V, eps, m->X_in[0], m->err_word, m->xn, amode, eps);
-  m->launches += 2;
+  m->launches += 1;
   const KVCacheView cv = cache_view(m);
   const int causal = fam != ADEPT_FAMILY_BERT;
   // generation step: the split-KV attention grid covers the reserved capacity (CTAs past a
@@ -1873,11 +1878,14 @@ adept_status adept_decode_step(adept_model* m, int batch, const int32_t* d_token
   }
   cudaStream_t st = (cudaStream_t)stream;
   // inputs into the staging buffers; the step itself reads and writes only those
-  launch_stage_in(st, m->d_delta, delta, d_tokens, m->dec_tok, d_forced_exit, m->dec_forced, batch);
+  launch_step_in(st, m->d_delta, delta, d_tokens, m->dec_tok, d_forced_exit, m->dec_forced, batch, m->tok_seq, m->tok_pos,
+                 m->row_tok[0], m->d_seq_len, m->max_blocks_per_seq * m->cfg.kv_block_tokens,
+                 m->cfg.family == ADEPT_FAMILY_LLAMA ? 0 : m->cfg.max_pos, m->err_word, m->ctr, ctr_words(m->N), m->dec_sim,
+                 m->N);
   m->launches += 1;
   auto body = [&](cudaStream_t s) -> adept_status {
     TRY(run_pass(m, batch, batch, 1, true, m->dec_tok, m->dec_forced, m->dec_exit, m->dec_sim, s));
-    TRY(run_head(m, batch, 1, true, m->logits_ws, m->dec_next, s));
+    TRY(run_head(m, batch, 1, true, m->logits_ws, nullptr, s));
     span_collect(m, s);
     return ADEPT_OK;
   };
@@ -1911,10 +1919,10 @@ adept_status adept_decode_step(adept_model* m, int batch, const int32_t* d_token
     m->dec_warm[batch] += 1;
   }
   for (int b = 0; b < batch; ++b) m->h_seq_len[b] += 1;
-  // outputs out of the staging buffers, one launch
+  // outputs out of the staging buffers and the greedy tokens, one launch
   if (d_exit_layer_out || d_next_token_out || d_logits_out || d_sim_out) {
-    launch_stage_out(st, batch, m->dec_exit, d_exit_layer_out, m->dec_next, d_next_token_out, m->logits_ws,
-                     d_logits_out, (long long)batch * m->V, m->dec_sim, d_sim_out, batch * m->N);
+    launch_step_out(st, batch, m->V, m->logits_ws, d_logits_out, d_next_token_out, m->amax_v, m->amax_i, m->amax_cnt,
+                    m->dec_exit, d_exit_layer_out, m->dec_sim, d_sim_out, batch * m->N);
     m->launches += 1;
   }
   return check_launch(m);

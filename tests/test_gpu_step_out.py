@@ -1,0 +1,34 @@
+"""The last launch of a generation step: greedy tokens (the first of equal logits) and the copies of logits, exits and
+similarities, for vocabularies in one part and in many, over repeated steps and with outputs left out."""
+import pytest
+import torch
+
+import synth
+
+import paper_2601_03700_gb300 as adept
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("vocab", [1000, 4097, 50257])
+@pytest.mark.parametrize("batch", [1, 5])
+def test_step_outputs(vocab, batch):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    cfg = synth.ModelConfig(family=synth.GPT2, n_layers=3, d_model=128, n_heads=2, head_dim=64, d_ffn=256, vocab=vocab,
+                            max_pos=64, dtype="bf16", hsm_m1=256, hsm_m2=512, max_batch=batch, max_seq=32,
+                            max_pass_tokens=4 * batch)
+    W = synth.make_weights(cfg, seed=140, device="cuda")
+    W["tok_emb"][vocab // 2:] = W["tok_emb"][:vocab - vocab // 2].clone()   # equal rows: equal logits (tied head)
+    m = adept.Model(cfg, W)
+    m.prefill(synth.make_tokens(141, batch, 4, vocab).cuda(), 0.9)
+    tok = torch.zeros(batch, dtype=torch.int32, device="cuda")
+    for step in range(4):
+        ex, lg, nx, sims = m.decode_step(tok, 0.9)
+        want = (lg == lg.max(dim=1, keepdim=True).values).int().argmax(dim=1)
+        assert torch.equal(nx.long(), want)
+        assert int(ex.min()) >= 2 and int(ex.max()) <= 3 and sims.shape == (batch, 3)
+        adept.adept_decode_step(m.h, batch, tok, 0.9, next_token_out=nx)   # the others left out
+        tok = nx.clone()
+    m.check()
+    m.close()
