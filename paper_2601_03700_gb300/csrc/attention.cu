@@ -518,6 +518,13 @@ __device__ __forceinline__ bool ad_wait(uint64_t* bar, unsigned* err) {
 // a token that left at an earlier layer lets its copies land and leaves.  The copy barrier
 // takes two arrivals (before and after the wait), so it cannot complete between them.
 //
+// The grid covers the reserved capacity. Chunks past a token's keys leave at once, before the dependency wait, in a cluster too
+// (its barrier counts the CTAs that have not left, and the leader expects the others' partials only): when they stayed and pushed
+// empty partials they held SM slots that the next sequences' chunks waited for (16 sequences of 150 keys in a capacity of 512, 8 KV
+// heads: 512 CTAs for 456 slots; 6 steps of 4 layers 7.82 -> 7.65 ms with the 150-token prompt). A token whose keys lie in one chunk
+// keeps its whole cluster: with the leader alone a GPT-2-small turn of one sequence was slower in every run (6.46 against 6.57 ms),
+// whether the others left before the dependency wait or after it; the cause was not found.
+//
 // SV (one query head per KV head): the first half of the chunk's V rows has its own slots and
 // the second half is copied into the K slots once the scores are formed, so a CTA holds 1.5
 // chunks of rows instead of 2 (48 KB at d_h = 128): four CTAs fit on an SM and the grid of a
@@ -554,12 +561,14 @@ __global__ void __launch_bounds__(AD_THREADS)
                                                 // come from the pass's first kernel)
   const int sq = tok_seq[t], pos = tok_pos[t];
   const int nk = causal ? pos + 1 : seq_len[sq];
-  const int n_eff = (nk + AD_CHUNK - 1) / AD_CHUNK;   // chunks holding keys of this token
+  // chunks holding keys of this token
+  const int n_keyed = (nk + AD_CHUNK - 1) / AD_CHUNK;
+  const int n_eff = CL && n_keyed <= 1 ? n_split : n_keyed;   // the chunks that stay (see above)
   if (SV && group != 1) {   // (uniform over the grid) the K slots would be needed again
     if (tid == 0) atomicOr(err, ERRW_CONFIG);
     return;
   }
-  if (!CL && split >= n_eff) return;   // (a cluster's CTAs all stay: they push empty partials)
+  if (split >= n_eff) return;   // (a cluster's barrier waits for its CTAs that have not left)
   const int k_lo = split * AD_CHUNK, nkc = max(0, min(nk - k_lo, AD_CHUNK));
   const int nb = (nkc + 15) >> 4;                      // cache blocks of the chunk
   // blocks of the chunk below the block of the token's own position: written before this step
@@ -577,7 +586,7 @@ __global__ void __launch_bounds__(AD_THREADS)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     if (CL && split == 0)
       asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(ad_smem_u32(&red_bar)),
-                   "r"((uint32_t)(group * (n_split - 1) * PW * 4))
+                   "r"((uint32_t)(group * (n_eff - 1) * PW * 4))
                    : "memory");
   }
   __syncthreads();
@@ -915,10 +924,10 @@ __global__ void __launch_bounds__(AD_THREADS)
       const int h = kvh * group + g;
       const float* sl = sPart + (size_t)g * n_split * PW;
       float Mg = -INFINITY;
-      for (int c = 0; c < n_split; ++c) Mg = fmaxf(Mg, sl[c * PW + DH]);
+      for (int c = 0; c < n_eff; ++c) Mg = fmaxf(Mg, sl[c * PW + DH]);
       float L = 0.f, acc = 0.f;
       const int d = tid;
-      for (int c = 0; c < n_split; ++c) {
+      for (int c = 0; c < n_eff; ++c) {
         const float m = sl[c * PW + DH];
         if (m == -INFINITY) continue;
         const float sc = exp2f(m - Mg);
