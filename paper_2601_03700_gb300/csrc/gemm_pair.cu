@@ -17,10 +17,10 @@
 // Measured against the one-CTA tiles of 128 rows x 256 or 128 columns (gemm_tc.cu), which loaded 48 KB per k-block and SM (about
 // 68 bytes per clock, the most seen) and ended in a last wave of a few tiles. 2048 rows: 12288 x 4096 144 -> 115 us (1.79
 // PFLOP/s), 22016 x 4096 228 -> 200, 4096 x 11008 143 -> 105, 4096 x 4096 67 -> 50; 680 rows x 8192 x 32768 419 -> 259;
-// 8192 rows x 768 x 768 with residual 36 -> 22, x 3072 x 768 with GELU 73 -> 45. Bound by the tensor cores from K of about 2000 on (0.9 of their rate at the
-// chosen width), by the epilogue's turn-around and stores below that.
+// 8192 rows x 768 x 768 with residual 36 -> 22, x 3072 x 768 with GELU 73 -> 45. Bound by the tensor cores from K of about 2000
+// on (0.9 of their rate at the chosen width), by the epilogue's turn-around and stores below that.
 //
-// CTA = 10 warps: warp 0 lane 0 TMA producer; warp 1 tensor-memory allocator, its lane 0 in CTA 0 issues the pair's MMAs;
+// CTA = 10 warps: one thread of warp 0 TMA producer; warp 1 tensor-memory allocator, one of its threads in CTA 0 issues the pair's MMAs;
 // warps 2..9 epilogue. Ring of k-blocks with full barriers in CTA 0 (both CTAs' copies complete on it) and empty barriers in
 // both; two accumulator buffers. Waits are bounded: on time-out a CTA sets ERRW_TIMEOUT, stops, and leaves with its peer.
 #define ADEPT_TU_ID 12
