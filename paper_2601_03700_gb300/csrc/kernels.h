@@ -44,9 +44,14 @@ bool launch_embed_rows(cudaStream_t st, int dt, const int* tokens, int n_tok, co
                        float eps, float* X, unsigned* err, void* xhat, int smode, float seps);
 void launch_standardize(cudaStream_t st, int dt, const float* X, int ldx, const int* in_rows, DevRange rows,
                         int max_rows, int D, int mode, float eps, void* out, int ld_out);
-// LayerNorm with gain and shift of rows of X in place, and the result in the model's type in xt.
+// LayerNorm with gain and shift of rows of X in place, and the result in the model's type in xt (optional).
 void launch_layernorm_rows(cudaStream_t st, int dt, float* X, DevRange rows, int max_rows, int D, const float* g,
                            const float* b, float eps, void* xt);
+// The same with the exit test of the rows (X = s_i); false (nothing launched) for rows above 8192 elements.
+bool launch_layernorm_exit_test(cudaStream_t st, float* X, DevRange rows, int max_rows, int D, const float* g, const float* b,
+                                float eps, const float* Xin, const float* I, const int* row_tok, const int* forced,
+                                int layer, int n_layers, const float* delta_p, int test, int metric, float* sim, int* flag,
+                                float* inv_norm, unsigned* err);
 // The exit step of a layer: test, inertia update, stable compaction, and the kept rows
 // standardised (smode, seps) as the next layer's attention input, in the model's type, in
 // xhat_next.  metric: EXIT_*; Xin = the layer's input rows s_{i-1}.  aao_len: all-at-once prompt
@@ -54,7 +59,9 @@ void launch_layernorm_rows(cudaStream_t st, int dt, float* X, DevRange rows, int
 // prompt token; tok_pos gives a token's position), 0 = token level.  max_rows: the pass's row
 // bound.  launch_exit_decode: one CTA that holds every row in registers; returns false (nothing
 // launched) above 16 rows or rows that its registers do not hold (at D = 4096, above 4 rows).
-// launch_exit_rows: two launches over any number of rows (flag, inv_norm: one word per row).
+// launch_exit_rows: two launches over any number of rows (flag, inv_norm: one word per row); one where
+// launch_layernorm_exit_test has filled flag, inv_norm and sim (tested).
+bool exit_decode_takes(int max_rows, int D);   // what launch_exit_decode holds
 bool launch_exit_decode(cudaStream_t st, int dt, const float* Xin, const float* Xout, const float* I, int first, int D,
                         int* ctr, int par, const int* row_tok, int* row_tok_next, const int* forced, int layer,
                         int n_layers, const float* delta_p, int test, float* sim, int* exit_tok, int* exit_layer_out,
@@ -66,7 +73,7 @@ void launch_exit_rows(cudaStream_t st, int dt, const float* Xin, const float* Xo
                       int layer, int n_layers, const float* delta_p, int test, int metric, float* sim, int* flag,
                       float* inv_norm, int* exit_tok, int* exit_layer_out, float* Xnext, float* Inext, float* hsm_s,
                       float* hsm_prev, float* hsm_I, void* xhat, int smode, float seps, int aao_len,
-                      const int* tok_pos, unsigned* err);
+                      const int* tok_pos, unsigned* err, bool tested);
 void launch_set_float(cudaStream_t st, float* p, float v);
 void launch_span_collect(cudaStream_t st, SpanSite* sites, int n, SpanTotal* tot, int n_cls);
 // Generation-step staging of the caller's inputs (forced NULL -> zeros) with the pass's set-up, and of the

@@ -338,15 +338,21 @@ __global__ void __launch_bounds__(EXD_THREADS)
   }
 }
 
+bool exit_decode_takes(int max_rows, int D) {
+  int rshift = 0;
+  while ((1 << rshift) < max_rows) ++rshift;
+  return max_rows <= 16 && D / 4 <= EXD_V * (EXD_THREADS >> rshift);
+}
+
 bool launch_exit_decode(cudaStream_t st, int dt, const float* Xin, const float* Xout, const float* I, int first, int D,
                         int* ctr, int par, const int* row_tok, int* row_tok_next, const int* forced, int layer,
                         int n_layers, const float* delta_p, int test, float* sim, int* exit_tok, int* exit_layer_out,
                         float* Xnext, float* Inext, float* hsm_s, float* hsm_prev, float* hsm_I, int max_rows,
                         void* xhat_next, int smode, float seps, int metric, int aao_len, const int* tok_pos,
                         unsigned* err) {
+  if (!exit_decode_takes(max_rows, D)) return false;
   int rshift = 0;
   while ((1 << rshift) < max_rows) ++rshift;
-  if (max_rows > 16 || D / 4 > EXD_V * (EXD_THREADS >> rshift)) return false;
   const bool small = D / 4 <= 2 * (EXD_THREADS >> rshift);
 #define GO(V, T)                                                                                                     \
   launch_k(exit_decode_kernel<V, T>, 1, EXD_THREADS, 0, st, Xin, Xout, I, first, D, ctr, par, row_tok, row_tok_next, \

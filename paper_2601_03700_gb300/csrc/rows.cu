@@ -140,14 +140,40 @@ __global__ void __launch_bounds__(RW_THREADS)
   }
 }
 
+// The exit test of row r (token tok) from its sums |s_i|^2, |I|^2, <s_i, I>, |s_{i-1}|^2, <s_i, s_{i-1}>.
+struct ExitTest {
+  const int *row_tok, *forced;
+  int layer, n_layers, test, metric;
+  const float* delta;
+  float* sim;
+  int* flag;
+  float* inv_norm;
+  unsigned* err;
+};
+__device__ __forceinline__ void exit_decide(const ExitTest& t, int r, int tok, const float (&a)[5]) {
+  int ex = 0;
+  if (t.test) {
+    const float c = exit_similarity(t.metric, a[0], a[1], a[2], a[3], a[4]);
+    if (t.sim) t.sim[(size_t)tok * t.n_layers + (t.layer - 1)] = c;
+    const int f = t.forced ? t.forced[tok] : 0;
+    if (f != 0 && (f < 2 || f > t.n_layers)) atomicOr(t.err, ERRW_FORCED);
+    ex = (f > 0) ? (f == t.layer) : (c >= *t.delta);
+  }
+  t.flag[r] = ex;
+  t.inv_norm[r] = a[0] > 0.f ? rsqrtf(a[0]) : 0.f;
+}
+
 // The post-LN encoder's residual stream: LayerNorm with gain and shift in place, and the result
-// as the next product's operand in the model's type (xt, row stride D).
-template <typename T, int TPR, int V>
+// as the next product's operand in the model's type (xt, optional, row stride D).
+// TEST (V > 0): the layer's last LayerNorm, which also takes the exit test of the row while it is
+// held (the test on its own read the row again and took a launch: 9.3 us for 8192 rows of 768).
+template <typename T, int TPR, int V, bool TEST>
 __global__ void __launch_bounds__(RW_THREADS)
     layernorm_rows_kernel(float* __restrict__ X, DevRange rows, int D, const float* __restrict__ g,
-                          const float* __restrict__ b, float eps, T* __restrict__ xt) {
+                          const float* __restrict__ b, float eps, T* __restrict__ xt, const float* __restrict__ I,
+                          const float* __restrict__ Xin, ExitTest t) {
   PDL_ENTRY();
-  __shared__ float red[RW_THREADS / 32];
+  __shared__ float red[RW_THREADS / 32 * (TEST ? 5 : 1)];
   constexpr int G = RW_THREADS / TPR;
   const int rb = rows.b(), re = rows.e(), D4 = D >> 2, sub = threadIdx.x & (TPR - 1);
   for (int r = rb + blockIdx.x * G + (int)threadIdx.x / TPR; r < re; r += gridDim.x * G) {
@@ -156,17 +182,42 @@ __global__ void __launch_bounds__(RW_THREADS)
 #pragma unroll
     for (int j = 0; j < V; ++j)
       if (sub + j * TPR < D4) x[j] = row4(src, sub + j * TPR, true);
+    float4 c[TEST ? V : 1];
+    if (TEST && t.test) {
+#pragma unroll
+      for (int j = 0; j < V; ++j)
+        if (sub + j * TPR < D4) c[j] = row4(I + (size_t)r * D, sub + j * TPR, true);
+    }
     const float2 n = row_norm<TPR, V>(x, src, true, sub, D4, D, NORM_LN, eps, red);
     auto out = [&](int v, float4 a) {
       const float4 c = scale4(centre4(a, n.x), n.y), gg = row4(g, v, true), bb = row4(b, v, true);
       const float4 y = make_float4(c.x * gg.x + bb.x, c.y * gg.y + bb.y, c.z * gg.z + bb.z, c.w * gg.w + bb.w);
       put4(src, v, y);
-      put4(xt + (size_t)r * D, v, y);
+      if (xt) put4(xt + (size_t)r * D, v, y);
+      return y;
     };
     if (V) {
+      float a[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-      for (int j = 0; j < V; ++j)
-        if (sub + j * TPR < D4) out(sub + j * TPR, x[j]);
+      for (int j = 0; j < V; ++j) {
+        if (sub + j * TPR >= D4) continue;
+        const float4 y = out(sub + j * TPR, x[j]);
+        if (!TEST) continue;
+        a[0] += dot4(y, y);
+        if (t.test) {   // layer 1 tests nothing: only its norm is needed
+          a[1] += dot4(c[j], c[j]);
+          a[2] += dot4(y, c[j]);
+          if (t.metric != EXIT_GLOBAL) {
+            const float4 s = row4(Xin + (size_t)r * D, sub + j * TPR, true);
+            a[3] += dot4(s, s);
+            a[4] += dot4(y, s);
+          }
+        }
+      }
+      if (TEST) {
+        group_sum<TPR, 5>(a, red);
+        if (sub == 0) exit_decide(t, r, t.row_tok[r], a);
+      }
     } else {
       for (int v = sub; v < D4; v += TPR) out(v, row4(src, v, true));   // a thread rewrites only what it reads
     }
@@ -179,9 +230,7 @@ __global__ void __launch_bounds__(RW_THREADS)
 template <int TPR>
 __global__ void __launch_bounds__(RW_THREADS)
     exit_decide_kernel(const float* __restrict__ Xout, const float* __restrict__ I, const float* __restrict__ Xin,
-                       int D, DevRange rows, const int* row_tok, const int* forced, int layer, int n_layers,
-                       const float* delta_p, int test, int metric, float* sim, int* flag, float* inv_norm,
-                       unsigned* err) {
+                       int D, DevRange rows, ExitTest t) {
   PDL_ENTRY();
   __shared__ float red[RW_THREADS / 32 * 5];
   const int r = blockIdx.x * (RW_THREADS / TPR) + (int)threadIdx.x / TPR, sub = threadIdx.x & (TPR - 1);
@@ -189,18 +238,18 @@ __global__ void __launch_bounds__(RW_THREADS)
   const float4* s = reinterpret_cast<const float4*>(Xout + (size_t)r * D);
   const float4* in = reinterpret_cast<const float4*>(I + (size_t)r * D);
   const float4* sp = reinterpret_cast<const float4*>(Xin + (size_t)r * D);
-  const int tok = row_tok[r];
+  const int tok = t.row_tok[r];
   float a[5] = {0.f, 0.f, 0.f, 0.f, 0.f};   // |s_i|^2, |I|^2, <s_i, I>, |s_{i-1}|^2, <s_i, s_{i-1}>
   const int D4 = D >> 2;
 #pragma unroll 4
   for (int v = sub; v < D4; v += TPR) {
     const float4 x = s[v];
     a[0] += dot4(x, x);
-    if (test) {   // layer 1 tests nothing: only its norm is needed
+    if (t.test) {   // layer 1 tests nothing: only its norm is needed
       const float4 c = in[v];
       a[1] += dot4(c, c);
       a[2] += dot4(x, c);
-      if (metric != EXIT_GLOBAL) {
+      if (t.metric != EXIT_GLOBAL) {
         const float4 b = sp[v];
         a[3] += dot4(b, b);
         a[4] += dot4(x, b);
@@ -209,16 +258,7 @@ __global__ void __launch_bounds__(RW_THREADS)
   }
   group_sum<TPR, 5>(a, red);
   if (sub != 0) return;
-  int ex = 0;
-  if (test) {
-    const float c = exit_similarity(metric, a[0], a[1], a[2], a[3], a[4]);
-    if (sim) sim[(size_t)tok * n_layers + (layer - 1)] = c;
-    const int f = forced ? forced[tok] : 0;
-    if (f != 0 && (f < 2 || f > n_layers)) atomicOr(err, ERRW_FORCED);
-    ex = (f > 0) ? (f == layer) : (c >= *delta_p);
-  }
-  flag[r] = ex;
-  inv_norm[r] = a[0] > 0.f ? rsqrtf(a[0]) : 0.f;
+  exit_decide(t, r, tok, a);
 }
 
 // The compaction and the moves in one launch.  A CTA takes an equal run of the active rows; it
@@ -426,12 +466,27 @@ void launch_standardize(cudaStream_t st, int dt, const float* X, int ldx, const 
 void launch_layernorm_rows(cudaStream_t st, int dt, float* X, DevRange rows, int max_rows, int D, const float* g,
                            const float* b, float eps, void* xt) {
   if (max_rows <= 0) return;
-#define GO(T, TPR, V)                                                                                             \
-  launch_k(layernorm_rows_kernel<T, TPR, V>, rows_grid(max_rows, RW_THREADS / TPR), RW_THREADS, 0, st, X, rows, D, \
-           g, b, eps, (T*)xt)
+#define GO(T, TPR, V)                                                                                                    \
+  launch_k(layernorm_rows_kernel<T, TPR, V, false>, rows_grid(max_rows, RW_THREADS / TPR), RW_THREADS, 0, st, X, rows, D, \
+           g, b, eps, (T*)xt, (const float*)nullptr, (const float*)nullptr, ExitTest{})
   if (dt == 1) ROWS_DISPATCH(bf16, D, GO);
   else ROWS_DISPATCH(float, D, GO);
 #undef GO
+}
+
+bool launch_layernorm_exit_test(cudaStream_t st, float* X, DevRange rows, int max_rows, int D, const float* g, const float* b,
+                                float eps, const float* Xin, const float* I, const int* row_tok, const int* forced,
+                                int layer, int n_layers, const float* delta_p, int test, int metric, float* sim, int* flag,
+                                float* inv_norm, unsigned* err) {
+  if (D > 8192) return false;   // (such rows are not held)
+  if (max_rows <= 0) return true;
+  const ExitTest t{row_tok, forced, layer, n_layers, test, metric, delta_p, sim, flag, inv_norm, err};
+#define GO(T, TPR, V)                                                                                                     \
+  launch_k(layernorm_rows_kernel<T, TPR, V ? V : 8, true>, rows_grid(max_rows, RW_THREADS / TPR), RW_THREADS, 0, st, X, rows, \
+           D, g, b, eps, (T*)nullptr, I, Xin, t)
+  ROWS_DISPATCH(float, D, GO);
+#undef GO
+  return true;
 }
 
 void launch_exit_rows(cudaStream_t st, int dt, const float* Xin, const float* Xout, const float* I, int first, int D,
@@ -439,15 +494,16 @@ void launch_exit_rows(cudaStream_t st, int dt, const float* Xin, const float* Xo
                       int layer, int n_layers, const float* delta_p, int test, int metric, float* sim, int* flag,
                       float* inv_norm, int* exit_tok, int* exit_layer_out, float* Xnext, float* Inext, float* hsm_s,
                       float* hsm_prev, float* hsm_I, void* xhat, int smode, float seps, int aao_len,
-                      const int* tok_pos, unsigned* err) {
+                      const int* tok_pos, unsigned* err, bool tested) {
   if (max_rows <= 0) return;
   const DevRange act{nullptr, ctr + CTR_ACTIVE + par, 0};
-  if (D <= 1024)
-    launch_k(exit_decide_kernel<32>, cdiv(max_rows, RW_THREADS / 32), RW_THREADS, 0, st, Xout, I, Xin, D, act, row_tok,
-             forced, layer, n_layers, delta_p, test, metric, sim, flag, inv_norm, err);
-  else
-    launch_k(exit_decide_kernel<256>, max_rows, RW_THREADS, 0, st, Xout, I, Xin, D, act, row_tok, forced, layer,
-             n_layers, delta_p, test, metric, sim, flag, inv_norm, err);
+  const ExitTest t{row_tok, forced, layer, n_layers, test, metric, delta_p, sim, flag, inv_norm, err};
+  if (tested) {
+  } else if (D <= 1024) {
+    launch_k(exit_decide_kernel<32>, cdiv(max_rows, RW_THREADS / 32), RW_THREADS, 0, st, Xout, I, Xin, D, act, t);
+  } else {
+    launch_k(exit_decide_kernel<256>, max_rows, RW_THREADS, 0, st, Xout, I, Xin, D, act, t);
+  }
 #define GO(T, TPR, V)                                                                                              \
   launch_k(exit_move_kernel<T, TPR, V>, rows_grid(max_rows, TPR == 32 ? 4 : 1), RW_THREADS, 0, st, Xin, Xout, I,   \
            first, D, ctr, par, flag, inv_norm, row_tok, row_tok_next, exit_tok, exit_layer_out, layer, Xnext, Inext, \

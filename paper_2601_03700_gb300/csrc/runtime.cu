@@ -1123,6 +1123,7 @@ static adept_status run_pass(adept_model* m, int n_tok, int batch, int prompt_le
   } pend = {false, 0, 0, nullptr, nullptr, nullptr};
   // the exit step of layer `layer` on its own: one CTA that holds the rows where it can, else two
   // launches over the rows
+  bool tested = false;   // the layer's exit test was part of its last LayerNorm (encoder)
   auto exit_step = [&](int layer, int p, float* Xi, float* Ii, int* rt) {
     const int test = layer >= 2;
     if (launch_exit_decode(st, m->dt, Xi, m->X_out, Ii, layer == 1, D, m->ctr, p, rt, m->row_tok[p ^ 1], forced, layer,
@@ -1135,8 +1136,8 @@ static adept_status run_pass(adept_model* m, int n_tok, int batch, int prompt_le
     launch_exit_rows(st, m->dt, Xi, m->X_out, Ii, layer == 1, D, m->ctr, p, n_tok, rt, m->row_tok[p ^ 1], forced, layer,
                      N, m->d_delta, test, m->exit_metric, sim_out, m->flag, m->inv_norm, m->exit_tok, exit_w,
                      m->X_in[p ^ 1], m->I[p ^ 1], m->hsm_s, m->hsm_prev, m->hsm_I, m->xn, amode, eps, aao_len,
-                     m->tok_pos, m->err_word);
-    m->launches += 2;
+                     m->tok_pos, m->err_word, tested);
+    m->launches += tested ? 1 : 2;
   };
   int par = 0;
   for (int i = 1; i <= N; ++i) {
@@ -1269,7 +1270,12 @@ static adept_status run_pass(adept_model* m, int n_tok, int batch, int prompt_le
     p.epi.resid = m->X_out; p.epi.ld_resid = D;
     gemm(m, st, &p, 1, &mr, m->gemm_cls);
     if (fam == ADEPT_FAMILY_BERT) {
-      launch_layernorm_rows(st, m->dt, m->X_out, act, mr, D, w.ln2_g, w.ln2_b, eps, m->xn);
+      // s_i (the exit step, or the last layer's scatter, makes the next operand of it), with the exit test where that
+      // step does not hold the rows
+      tested = i < N && !exit_decode_takes(mr, D) &&
+               launch_layernorm_exit_test(st, m->X_out, act, mr, D, w.ln2_g, w.ln2_b, eps, Xi, Ii, rt, forced, i, N,
+                                          m->d_delta, i >= 2, m->exit_metric, sim_out, m->flag, m->inv_norm, m->err_word);
+      if (!tested) launch_layernorm_rows(st, m->dt, m->X_out, act, mr, D, w.ln2_g, w.ln2_b, eps, nullptr);
       m->launches += 1;
     }
     if (i < N) {
