@@ -465,10 +465,18 @@ __global__ void __launch_bounds__(PG_THREADS, 1) gemm_pair_kernel(const __grid_c
             }
           }
         }
-        // every copy of the pair has landed before CTA 0 leaves (CTA 1 waits for it below)
+        // every copy of the pair has landed before CTA 0 leaves (CTA 1 waits for it below); after a time-out a stage may
+        // lack the other CTA's copies, and the time given below lets them land
         if (rank == 0)
-          for (int k = 0; k < S; ++k)
-            if (issued >> k & 1u) wait_fixed(&full[k], (last_par >> k) & 1u, p.err);
+          for (int k = 0; k < S; ++k) {
+            const long long t0 = clock64();
+            while ((issued >> k & 1u) && !mbar_try_wait(&full[k], (last_par >> k) & 1u) && !*abort_flag) {
+              if (clock64() - t0 > PG_TIMEOUT_CYCLES) {
+                atomicOr(p.err, ERRW_TIMEOUT);
+                *abort_flag = 1;
+              }
+            }
+          }
       }
     } else if (warp == 1) {
       if (rank == 0 && elect_one()) {

@@ -58,3 +58,21 @@ def test_pair_gemm_grouped_fill_matches_oracle(n):
         assert_rows_close(gk[pos[sel]], k, pair.tol, f"K layer {r}")
         assert_rows_close(gv[pos[sel]], v, pair.tol, f"V layer {r}")
     pair.close()
+
+
+def test_short_wait_limit_times_out_and_recovers():
+    """Waits that run out in a pass on the paired tiles: the status says so, the context stays usable, and with the limit
+    restored the same model matches the oracle."""
+    pair = Pair(config(synth.GPT2, 2, 150), seed=120)
+    tokens = synth.make_tokens(121, 2, 150, 1003).numpy()
+    forced = synth.forced_exits_uniform(122, 300, 2, 5).numpy().reshape(2, 150)
+    adept.adept_set_wait_limit(32)
+    try:
+        pair.gm.prefill(torch.as_tensor(tokens).cuda(), 0.9, torch.as_tensor(forced).cuda())
+        with pytest.raises(adept.AdeptError) as ei:
+            pair.gm.check()
+        assert ei.value.status == 5, str(ei.value)
+    finally:
+        adept.adept_set_wait_limit(0)
+    compare_prefill(pair, tokens, 0.9, forced)
+    pair.close()
