@@ -392,9 +392,10 @@ ADEPT_API int64_t adept_hsm_param_numel(const adept_model* m, int param);
  * ADEPT_ERR_TIMEOUT; the outputs of that call are undefined and the model stays usable.
  * Applies to every model of the process on the current device.  Errors: INVALID_ARG
  * (cycles < 0), CUDA.
- * adept_set_alloc_fail_after: after n more device allocations by the library, every further
- * allocation fails as if the device were out of memory (n < 0: off, the default); calls that
- * need memory then return ADEPT_ERR_OOM with everything they allocated released. */
+ * adept_set_alloc_fail_after: after n more device allocations by the library (making the graph of
+ * a generation step counts as one), every further allocation fails as if the device were out of
+ * memory (n < 0: off, the default); calls that need memory then return ADEPT_ERR_OOM with
+ * everything they allocated released, and can be made again. */
 ADEPT_API adept_status adept_set_wait_limit(int64_t cycles);
 ADEPT_API void adept_set_alloc_fail_after(int64_t n);
 

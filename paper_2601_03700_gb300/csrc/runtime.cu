@@ -217,14 +217,18 @@ static adept_status fail(adept_model* m, adept_status s, const char* fmt, ...) {
 // Allocation-failure hook (adept_set_alloc_fail_after): allocations left before every device
 // allocation of the library fails; negative: off.
 static std::atomic<long long> g_alloc_budget{-1};
+static bool alloc_refused() {
+  for (long long b = g_alloc_budget.load(); b >= 0;) {
+    if (b == 0) return true;
+    if (g_alloc_budget.compare_exchange_weak(b, b - 1)) break;
+  }
+  return false;
+}
 
 static adept_status dalloc(adept_model* m, void** p, size_t bytes) {
   *p = nullptr;
   if (bytes == 0) return ADEPT_OK;
-  for (long long b = g_alloc_budget.load(); b >= 0;) {
-    if (b == 0) return fail(m, ADEPT_ERR_OOM, "cudaMalloc(%zu) refused by the allocation-failure hook", bytes);
-    if (g_alloc_budget.compare_exchange_weak(b, b - 1)) break;
-  }
+  if (alloc_refused()) return fail(m, ADEPT_ERR_OOM, "cudaMalloc(%zu) refused by the allocation-failure hook", bytes);
   cudaError_t e = cudaMalloc(p, bytes);
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -1883,42 +1887,51 @@ adept_status adept_decode_step(adept_model* m, int batch, const int32_t* d_token
       return fail(m, ADEPT_ERR_CAPACITY, "sequence %d is full (%d positions)", b, m->h_seq_len[b]);
   }
   cudaStream_t st = (cudaStream_t)stream;
-  // inputs into the staging buffers; the step itself reads and writes only those
-  launch_step_in(st, m->d_delta, delta, d_tokens, m->dec_tok, d_forced_exit, m->dec_forced, batch, m->tok_seq, m->tok_pos,
-                 m->row_tok[0], m->d_seq_len, m->max_blocks_per_seq * m->cfg.kv_block_tokens,
-                 m->cfg.family == ADEPT_FAMILY_LLAMA ? 0 : m->cfg.max_pos, m->err_word, m->ctr, ctr_words(m->N), m->dec_sim,
-                 m->N);
-  m->launches += 1;
   auto body = [&](cudaStream_t s) -> adept_status {
     TRY(run_pass(m, batch, batch, 1, true, m->dec_tok, m->dec_forced, m->dec_exit, m->dec_sim, s));
     TRY(run_head(m, batch, 1, true, m->logits_ws, nullptr, s));
     span_collect(m, s);
     return ADEPT_OK;
   };
-  const bool graph_ok = m->use_graph && !m->profile;
-  if (graph_ok && m->dec_warm[batch] >= 1) {
-    if (!m->dec_graph[batch]) {
-      // capture one generation step on a private stream; later steps replay it
-      if (!m->cap_stream) CUDA_TRY(m, cudaStreamCreateWithFlags(&m->cap_stream, cudaStreamNonBlocking));
-      const int64_t l0 = m->launches;
-      CUDA_TRY(m, cudaStreamBeginCapture(m->cap_stream, cudaStreamCaptureModeThreadLocal));
-      adept_status s = body(m->cap_stream);
-      cudaGraph_t g = nullptr;
-      cudaError_t e = cudaStreamEndCapture(m->cap_stream, &g);
-      if (s != ADEPT_OK) {
-        if (g) cudaGraphDestroy(g);
-        return s;
-      }
-      if (e != cudaSuccess) return fail(m, ADEPT_ERR_CUDA, "graph capture failed: %s", cudaGetErrorString(e));
-      cudaGraphExec_t ex = nullptr;
-      e = cudaGraphInstantiate(&ex, g, 0);
-      cudaGraphDestroy(g);
-      if (e != cudaSuccess) return fail(m, ADEPT_ERR_CUDA, "graph instantiate failed: %s", cudaGetErrorString(e));
-      m->dec_graph[batch] = ex;
-      m->graph_launches = m->launches - l0;
-      m->launches = l0;
+  // The graph first: a step that cannot be captured has launched nothing, and the call can be made again.
+  const bool replay = m->use_graph && !m->profile && m->dec_warm[batch] >= 1;
+  if (replay && !m->dec_graph[batch]) {
+    // capture one generation step on a private stream; later steps replay it
+    if (!m->cap_stream) CUDA_TRY(m, cudaStreamCreateWithFlags(&m->cap_stream, cudaStreamNonBlocking));
+    const int64_t l0 = m->launches;
+    CUDA_TRY(m, cudaStreamBeginCapture(m->cap_stream, cudaStreamCaptureModeThreadLocal));
+    adept_status s = body(m->cap_stream);
+    m->graph_launches = m->launches - l0;
+    m->launches = l0;
+    cudaGraph_t g = nullptr;
+    cudaError_t e = cudaStreamEndCapture(m->cap_stream, &g);
+    cudaGraphExec_t ex = nullptr;
+    if (s == ADEPT_OK && e != cudaSuccess) s = fail(m, ADEPT_ERR_CUDA, "graph capture failed: %s", cudaGetErrorString(e));
+    if (s == ADEPT_OK && alloc_refused())
+      s = fail(m, ADEPT_ERR_OOM, "cudaGraphInstantiate refused by the allocation-failure hook");
+    if (s == ADEPT_OK && (e = cudaGraphInstantiate(&ex, g, 0)) != cudaSuccess)
+      s = fail(m, ADEPT_ERR_CUDA, "graph instantiate failed: %s", cudaGetErrorString(e));
+    if (g) cudaGraphDestroy(g);
+    if (s != ADEPT_OK) {
+      cudaGetLastError();   // reported here; the next call starts clean
+      return s;
     }
-    CUDA_TRY(m, cudaGraphLaunch(m->dec_graph[batch], st));
+    m->dec_graph[batch] = ex;
+  }
+  // inputs into the staging buffers; the step itself reads and writes only those
+  launch_step_in(st, m->d_delta, delta, d_tokens, m->dec_tok, d_forced_exit, m->dec_forced, batch, m->tok_seq, m->tok_pos,
+                 m->row_tok[0], m->d_seq_len, m->max_blocks_per_seq * m->cfg.kv_block_tokens,
+                 m->cfg.family == ADEPT_FAMILY_LLAMA ? 0 : m->cfg.max_pos, m->err_word, m->ctr, ctr_words(m->N), m->dec_sim,
+                 m->N);
+  m->launches += 1;
+  if (replay) {
+    const cudaError_t e = cudaGraphLaunch(m->dec_graph[batch], st);
+    if (e != cudaSuccess) {
+      // the set-up has run and the step has not: the lengths as they were
+      cudaGetLastError();
+      cudaMemcpyAsync(m->d_seq_len, m->h_seq_len.data(), batch * sizeof(int), cudaMemcpyHostToDevice, st);
+      return fail(m, ADEPT_ERR_CUDA, "graph launch failed: %s", cudaGetErrorString(e));
+    }
     m->launches += m->graph_launches;
   } else {
     TRY(body(st));

@@ -6,8 +6,9 @@
   report ADEPT_ERR_TIMEOUT through adept_check_device_status, the context must stay usable,
   and with the limit restored the same model and a fresh one must match the oracle.
 * Device allocation failure: adept_set_alloc_fail_after makes the library's device
-  allocations fail from a chosen point on; model loading and the fill workspace's growth must
-  return ADEPT_ERR_OOM, release what they allocated, and leave the library usable."""
+  allocations fail from a chosen point on; model loading, the fill workspace's growth and the
+  graph of a generation step must return ADEPT_ERR_OOM, release what they allocated, and leave
+  the library usable."""
 import numpy as np
 import pytest
 import torch
@@ -128,3 +129,30 @@ def test_allocation_failure_returns_oom_and_releases_memory():
     torch.cuda.synchronize()
     free1 = torch.cuda.mem_get_info()[0]
     assert abs(free1 - free0) < (64 << 20), f"device memory not released: {(free0 - free1) / 2**20:.1f} MiB"
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_refused_step_graph_leaves_the_sequences_as_they_were(dtype):
+    """A generation step whose graph cannot be made has changed nothing: the same step made again, and those after it,
+    match the oracle, the cached K/V of every position among them."""
+    cfg = synth.ModelConfig(family=synth.LLAMA, n_layers=4, d_model=128, n_heads=2, head_dim=64, d_ffn=256, vocab=500,
+                            dtype=dtype, max_batch=3, max_seq=32, hsm_m1=256, hsm_m2=512, block_shuffle_seed=4)
+    pair = Pair(cfg, seed=54)
+    tokens = synth.make_tokens(54, 3, 5, cfg.vocab).numpy()
+    forced = synth.forced_exits_uniform(54, 15, 2, cfg.n_layers).numpy().reshape(3, 5)
+    ores, cache, _ = compare_prefill(pair, tokens, 0.9, forced)
+    steps = synth.forced_exits_uniform(55, 12, 2, cfg.n_layers).numpy().reshape(4, 3)
+    compare_decode(pair, cache, ores.next_token, 1, 0.9, steps[:1])   # the second step of a batch makes the graph
+    tok = ores.next_token * 0 + 7
+    adept.adept_set_alloc_fail_after(0)
+    try:
+        for _ in range(2):
+            with pytest.raises(adept.AdeptError) as ei:
+                pair.gm.decode_step(torch.as_tensor(tok, dtype=torch.int32).cuda(), 0.9,
+                                    torch.as_tensor(steps[1], dtype=torch.int32).cuda())
+            assert ei.value.status == OOM and "allocation-failure hook" in str(ei.value)
+    finally:
+        adept.adept_set_alloc_fail_after(-1)
+    compare_decode(pair, cache, tok, 3, 0.9, steps[1:])
+    pair.compare_cache(cache, 3, 9)
+    pair.close()
