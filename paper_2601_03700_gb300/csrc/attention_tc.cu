@@ -234,7 +234,6 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   pdl_wait();   // Q rows, row maps and the cache come from the preceding kernels
-  pdl_launch_dependents();
   // this CTA's tile, heads h0 .. h0 + nh and sequences z, z + Z, ..
   const int rbeg = p.rows.b(), rend = p.rows.e();
   const int tiles = (max(0, rend - rbeg) + AT_BM - 1) / AT_BM, Z = p.z;
@@ -263,6 +262,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_launch_dependents();   // after the TMEM allocation: a dependent CTA cannot take it first
   // runs of one sequence (rows are in sequence order) and each run's key range, in parallel:
   // thread = row; a run's index is the count of run starts up to its row
   __shared__ int s_wfirst[AT_BM / 32];
