@@ -22,7 +22,8 @@
 //
 // CTA = 10 warps: one thread of warp 0 TMA producer; warp 1 tensor-memory allocator, one of its threads in CTA 0 issues the pair's MMAs;
 // warps 2..9 epilogue. Ring of k-blocks with full barriers in CTA 0 (both CTAs' copies complete on it) and empty barriers in
-// both; two accumulator buffers. Waits are bounded: on time-out a CTA sets ERRW_TIMEOUT, stops, and leaves with its peer.
+// both; two accumulator buffers. Waits are bounded: on time-out a CTA sets ERRW_TIMEOUT and stops; the pair leaves together, once
+// every copy that either CTA issued has landed (pg_leave).
 #define ADEPT_TU_ID 12
 #include "gemm_pair.h"
 #include "epilogue.cuh"
@@ -52,7 +53,6 @@ constexpr int pg_width(int k) {
   return k == 0 ? 256 : k == 1 ? 224 : k == 2 ? 192 : k == 3 ? 160 : k == 4 ? 128 : k == 5 ? 96 : k == 6 ? 64 : 32;
 }
 constexpr long long PG_TIMEOUT_CYCLES = 4000000000LL;       // ~2 s at 2 GHz
-constexpr long long PG_LAND_CYCLES = 4000000LL;             // ~2 ms
 
 template <int MAXG>
 struct PgGroup {
@@ -113,6 +113,41 @@ __device__ __forceinline__ bool wait_fixed(uint64_t* bar, uint32_t par, unsigned
     }
   }
   return true;
+}
+
+// A word to this CTA's shared-memory address `local` in the pair's other CTA.
+__device__ __forceinline__ void put_peer(uint32_t local, int peer, uint32_t v) {
+  asm volatile("{\n.reg .b32 r;\nmapa.shared::cluster.u32 r, %0, %1;\nst.shared::cluster.u32 [r], %2;\n}\n" ::"r"(local), "r"(peer),
+               "r"(v)
+               : "memory");
+}
+__device__ __forceinline__ int pg_stage_bytes(int bn) { return PG_A_BYTES + bn * (PG_BK * 2 / 2); }
+__device__ __forceinline__ int pg_stages(int bn) { return min(PG_MAX_STAGES, PG_RING / pg_stage_bytes(bn)); }
+// A pair that stopped early (every thread of both CTAs): waits until all copies that they issued have landed. Both CTAs' copies
+// of a k-block complete on one barrier of CTA 0; a k-block that only one of them issued is given what the other did not send.
+// Out of line: a register kept for it in the main loops is one too many.
+__device__ __noinline__ void pg_leave(uint64_t* full, const uint32_t* issued, uint32_t* peer, int rank, int bn, unsigned* err) {
+  if (threadIdx.x == 0) put_peer(smem_u32(peer), rank ^ 1, *issued);
+  __syncwarp();
+  cluster_sync_all();
+  if (rank == 0 && threadIdx.x == 0) {
+    const uint32_t n0 = *issued, n1 = *peer, stage_bytes = (uint32_t)pg_stage_bytes(bn);
+    const int stages = pg_stages(bn);
+    const long long t0 = clock64();
+    bool ok = true;
+    for (int s = 0; s < stages && ok; ++s) {
+      const PgLanding l = pg_landing(n0, n1, (uint32_t)stages, (uint32_t)s);
+      if (l.owe == PgLanding::NOTHING) continue;
+      if (l.owe == PgLanding::ARRIVAL)
+        mbar_expect_tx(&full[s], stage_bytes);
+      else if (l.owe == PgLanding::BYTES)
+        asm volatile("mbarrier.complete_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&full[s])), "r"(stage_bytes) : "memory");
+      while (ok && !mbar_try_wait(&full[s], l.parity)) ok = clock64() - t0 <= PG_TIMEOUT_CYCLES;
+    }
+    if (!ok) atomicOr(err, ERRW_TIMEOUT);
+  }
+  __syncwarp();
+  cluster_sync_all();
 }
 
 // The time of one k-block of a tile in SM cycles: the MMAs take 2 BN (256 x BN x 64 at 8192 multiply-adds
@@ -335,6 +370,7 @@ __global__ void __launch_bounds__(PG_THREADS, 1) gemm_pair_kernel(const __grid_c
   __shared__ __align__(8) uint64_t full[PG_MAX_STAGES], empty[PG_MAX_STAGES], accf[2], acce[2], drain;
   __shared__ uint32_t tmem_slot;
   __shared__ int s_abort, s_bn, s_map;
+  __shared__ uint32_t s_issued, s_peer, s_stop;   // k-blocks whose copies this CTA issued; the other's; the other stopped early
   __shared__ int s_tile0[MAXG + 1], s_mbeg[MAXG], s_M[MAXG];
 
   const long long wlim = wait_limit();
@@ -356,6 +392,7 @@ __global__ void __launch_bounds__(PG_THREADS, 1) gemm_pair_kernel(const __grid_c
     }
     mbar_init(&drain, 1);
     s_abort = 0;
+    s_issued = s_stop = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&p.g[0].ta) : "memory");
   }
@@ -420,8 +457,8 @@ __global__ void __launch_bounds__(PG_THREADS, 1) gemm_pair_kernel(const __grid_c
   pdl_launch_dependents();
   const int BN = s_bn, total = s_tile0[ng];
   const uint32_t tmem = tmem_slot;
-  const int stage_bytes = PG_A_BYTES + BN * (PG_BK * 2 / 2);
-  const int S = min(PG_MAX_STAGES, PG_RING / stage_bytes);
+  const int stage_bytes = pg_stage_bytes(BN);
+  const int S = pg_stages(BN);
 
   // Tile order inside a problem: super-rows of gm m-tiles; within one n is the outer and m the inner index.
   auto locate = [&](int t, int& g, int& mb, int& nb) {
@@ -439,8 +476,8 @@ __global__ void __launch_bounds__(PG_THREADS, 1) gemm_pair_kernel(const __grid_c
       if (elect_one()) {
         // ------------------------------------------------------------ TMA producer (both CTAs)
         const uint32_t smem0 = smem_u32(smem), full0 = at_leader(smem_u32(full));
-        int s = 0, n_issued = 0;
-        uint32_t ph = 0, issued = 0, last_par = 0;
+        int s = 0;
+        uint32_t ph = 0, n_issued = 0;
         bool ok = true;
         for (int t = pair; t < total && ok; t += n_pairs) {
           int g, mb, nb;
@@ -450,33 +487,20 @@ __global__ void __launch_bounds__(PG_THREADS, 1) gemm_pair_kernel(const __grid_c
           const int ya = s_mbeg[g] + mb * PG_BM + rank * 128, yb = nb * BN + rank * (BN / 2);
           const CUtensorMap *ta = &G.ta, *tb = &G.tb[s_map];
           for (int kb = 0; kb < nk; ++kb) {
-            if (n_issued >= S && !(ok = mbar_wait(&empty[s], ph ^ 1, abort_flag, p.err, wlim))) break;
+            if (n_issued >= (uint32_t)S && !(ok = mbar_wait(&empty[s], ph ^ 1, abort_flag, p.err, wlim))) break;
             ++n_issued;
             const uint32_t bar = full0 + (uint32_t)s * 8;
             if (rank == 0) mbar_expect_tx(&full[s], (uint32_t)(2 * stage_bytes));
             const uint32_t dst = smem0 + (uint32_t)(s * stage_bytes);
             pair_load_2d(ta, bar, dst, kb * PG_BK, ya);
             pair_load_2d(tb, bar, dst + PG_A_BYTES, kb * PG_BK, yb);
-            issued |= 1u << s;
-            last_par = (last_par & ~(1u << s)) | (ph << s);
             if (++s == S) {
               s = 0;
               ph ^= 1;
             }
           }
         }
-        // every copy of the pair has landed before CTA 0 leaves (CTA 1 waits for it below); after a time-out a stage may
-        // lack the other CTA's copies, and the time given below lets them land
-        if (rank == 0)
-          for (int k = 0; k < S; ++k) {
-            const long long t0 = clock64();
-            while ((issued >> k & 1u) && !mbar_try_wait(&full[k], (last_par >> k) & 1u) && !*abort_flag) {
-              if (clock64() - t0 > PG_TIMEOUT_CYCLES) {
-                atomicOr(p.err, ERRW_TIMEOUT);
-                *abort_flag = 1;
-              }
-            }
-          }
+        s_issued = n_issued;
       }
     } else if (warp == 1) {
       if (rank == 0 && elect_one()) {
@@ -575,14 +599,11 @@ __global__ void __launch_bounds__(PG_THREADS, 1) gemm_pair_kernel(const __grid_c
       }
     }
   }
+  // The pair leaves together. Without a time-out every copy has landed: the MMAs that read it are through (drain).
   __syncthreads();
-  if (s_abort) {
-    // a CTA that stopped early has no barrier left that tells of its copies under way: they land within this time
-    const long long t0 = clock64();
-    while (clock64() - t0 < PG_LAND_CYCLES) {
-    }
-  }
-  cluster_sync_all();   // neither CTA touches the other any more
+  if (s_abort) put_peer(smem_u32(&s_stop), rank ^ 1, 1u);   // (by every thread)
+  cluster_sync_all();
+  if (s_abort || s_stop) pg_leave(full, &s_issued, &s_peer, rank, s_bn, p.err);   // (uniform over the pair)
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
@@ -700,6 +721,15 @@ int pair_gemm(cudaStream_t st, const GemmProblem* probs, int n_probs, const int*
     case EPI_RESID: return pg_go<EPI_RESID, 2>(st, probs, n_probs, err);
     case EPI_SWIGLU: return pg_go<EPI_SWIGLU, 2>(st, probs, n_probs, err);
     default: return pg_go<EPI_QKV, 2>(st, probs, n_probs, err);
+  }
+}
+
+// pg_landing of every stage: out[2 s] what is owed, out[2 s + 1] the parity to wait for.
+extern "C" __attribute__((visibility("default"))) void adept_debug_pair_landing(int n0, int n1, int stages, int* out) {
+  for (int s = 0; s < stages; ++s) {
+    const PgLanding l = pg_landing((uint32_t)n0, (uint32_t)n1, (uint32_t)stages, (uint32_t)s);
+    out[2 * s] = (int)l.owe;
+    out[2 * s + 1] = (int)l.parity;
   }
 }
 

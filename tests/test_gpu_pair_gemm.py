@@ -76,3 +76,30 @@ def test_short_wait_limit_times_out_and_recovers():
         adept.adept_set_wait_limit(0)
     compare_prefill(pair, tokens, 0.9, forced)
     pair.close()
+
+
+def test_waits_running_out_at_any_point_leave_the_pair_whole():
+    """Limits from a few cycles to a few microseconds stop the CTAs of a pair at different k-blocks, each with copies under
+    way that the other has not matched: every pass ends, says so in its status, and the next one is right."""
+    cfg = config(synth.GPT2, 3, 200, n_layers=3, d_model=1024, n_heads=16, d_ffn=4096, hsm_m1=2048, hsm_m2=4096)
+    pair = Pair(cfg, weights=synth.make_weights(cfg, seed=123, device="cuda"))
+    tokens = synth.make_tokens(124, 3, 200, 1003).numpy()
+    forced = synth.forced_exits_uniform(125, 600, 2, 3).numpy().reshape(3, 200)
+    dev = lambda x: torch.as_tensor(x).cuda()  # noqa: E731
+    pair.gm.prefill(dev(tokens), 0.9, dev(forced))
+    pair.gm.check()
+    stopped = 0
+    for limit in (1, 32, 200, 500, 1000, 1500, 2000, 3000, 5000, 10000):
+        adept.adept_set_wait_limit(limit)
+        try:
+            pair.gm.prefill(dev(tokens), 0.9, dev(forced))
+            try:
+                pair.gm.check()
+            except adept.AdeptError as e:
+                assert e.status == 5, str(e)
+                stopped += 1
+        finally:
+            adept.adept_set_wait_limit(0)
+    assert stopped >= 2
+    compare_prefill(pair, tokens, 0.9, forced)
+    pair.close()
