@@ -1,5 +1,5 @@
 // fp32-FMA GEMMs: the path of the fp32 models, and the cross-check of the tensor-core GEMM.
-// f32_rows_kernel (fp32, the epilogue fused) takes passes of up to F32_ROWS_MAX rows;
+// f32_rows_kernel (fp32, the epilogue fused) takes products of few rows (f32_rows_win);
 // gemm_simt_kernel, a 64 x 64 tile with a separate epilogue pass, the rest and bf16 operands (its
 // epilogue semantics are the reference for the fused tcgen05 epilogue).
 #define ADEPT_TU_ID 2
@@ -9,14 +9,36 @@
 
 namespace adept {
 
+// Whether f32_rows_kernel takes M rows of an N x K product, and not the 64 x 64 tiles.
+//
+// The rows kernel reads every weight again for each 8 rows and takes M N K / 6e12 s (K of up to 512, where a warp has one slice
+// of K, and above 8192, where a row's pieces leave L1 between features: M N K / 3.3e12 s); the tiles take 0.18 us per element of K
+// while they find a place on the SMs at once, then as many times more as there are tiles (a ninth of an SM each). Both
+// sides measured over 31 (N, K) from 256 x 256 to 32768 x 8192 and up to 256 rows: the better kernel is chosen in all but a
+// few places near the line, and there it is within 13 %. Bounds of 64 and 128 rows, rows kernel / tiles in us:
+// 4096 x 4096 197 / 738 and 370 / 715; 12288 x 4096 566 / 887 and 1118 / 989; 8192 x 16384 2499 / 3209 and 4994 / 3172;
+// 32768 x 8192 3006 / 2081 and 5641 / 3634. Prompt of 256 rows, D = 4096, FFN 11008, 4 layers, mapper 8192 / 16384: 37.1 ms on
+// the tiles alone, 44.9 on the rows kernel alone, 29.0 so. Up to 256 rows, as prompt passes of a model of D = 1024 (4 layers, mapper
+// 4096 / 8192), all rows to full depth, take 1.15 / 2.24 / 4.43 / 9.20 ms at 64 / 128 / 256 / 512 rows here and
+// 4.59 / 4.68 / 5.85 / 8.53 on the tiles.
+constexpr int F32_ROWS_MAX = 256;
+__host__ __device__ inline bool f32_rows_win(int M, int N, int K) {
+  if (M > F32_ROWS_MAX) return false;
+  const long long line = K > 512 && K <= 8192 ? 1100000 : 600000;   // outputs M N, while the tiles take one turn
+  const long long tiles = (long long)((N + 63) / 64) * ((M + 63) / 64), turn = 2432 + 5 * tiles;   // in 3040ths: 0.8 + tiles / 608
+  return (long long)M * N * 3040 <= line * (turn > 3040 ? turn : 3040);
+}
+
 // C[r, n] = sum_k A[begin + r, k] * B[n, k] for the rows of the problem's range.
 template <typename T>
 __global__ void __launch_bounds__(256) gemm_simt_kernel(const T* __restrict__ A, int lda, const T* __restrict__ B,
-                                                        int ldb, DevRange rows, int N, int K, float* C, int ldc) {
+                                                        int ldb, DevRange rows, int N, int K, float* C, int ldc,
+                                                        int above) {
   PDL_ENTRY();
   __shared__ float As[16][64 + 1];
   __shared__ float Bs[16][64 + 1];
   const int rb = rows.b(), M = rows.e() - rb;
+  if (above && f32_rows_win(M, N, K)) return;   // the rows kernel's
   const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
   if (m0 >= M) return;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -57,11 +79,11 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(const T* __restrict__ A,
 
 // Epilogue of one output row (see EpiKind), one thread per 32-column chunk.
 template <typename T>
-__global__ void epilogue_kernel(Epi e, const float* __restrict__ C, int ldc, DevRange rows, int N) {
+__global__ void epilogue_kernel(Epi e, const float* __restrict__ C, int ldc, DevRange rows, int N, int above, int K) {
   PDL_ENTRY();
   const int rb = rows.b(), M = rows.e() - rb;
   const int r = blockIdx.x;
-  if (r >= M) return;
+  if (r >= M || (above && f32_rows_win(M, N, K))) return;
   const int ra = rb + r;
   const float* c = C + (size_t)r * ldc;
   const EpiRow rr = epi_row(e, ra);
@@ -88,14 +110,11 @@ __global__ void epilogue_kernel(Epi e, const float* __restrict__ C, int ldc, Dev
 // 43 us a product on average plus 4 for its epilogue launch -> 2.3 to 5.0; its 64-token prompt and 16 steps 20.4 ->
 // 2.0 ms.
 constexpr int FR_THREADS = 256, FR_R = 8, FR_F = 4, FR_KC = 512;
-// The bound: prompt passes of a model of D = 1024 (4 layers, mapper 4096 / 8192), all rows to full depth, take
-// 1.15 / 2.24 / 4.43 / 9.20 ms at 64 / 128 / 256 / 512 rows here and 4.59 / 4.68 / 5.85 / 8.53 on the tile.
-constexpr int F32_ROWS_MAX = 256;
 
 template <int WK, int KIND>
 __global__ void __launch_bounds__(FR_THREADS) f32_rows_kernel(const float* __restrict__ A, int lda,
                                                               const float* __restrict__ B, int ldb, DevRange rows,
-                                                              int N, int K, Epi e, int ahead) {
+                                                              int N, int K, Epi e, int ahead, int below) {
   KT_BEGIN();
   constexpr int WF = FR_THREADS / 32 / WK, FT = FR_F * WF;   // feature groups, features of the CTA
   constexpr int NJ = FR_KC / 128;                            // float4 per lane of a slice
@@ -127,7 +146,7 @@ __global__ void __launch_bounds__(FR_THREADS) f32_rows_kernel(const float* __res
   KT_WAITED();
   pdl_launch_dependents();
   const int rb = rows.b(), M = rows.e() - rb, r0 = blockIdx.y * FR_R;
-  if (r0 >= M) return;
+  if (r0 >= M || (below && !f32_rows_win(M, N, K))) return;   // (below: more rows are the tiles')
   const int nr = min(FR_R, M - r0);
   float acc[FR_F * FR_R];
 #pragma unroll
@@ -213,12 +232,12 @@ __global__ void __launch_bounds__(FR_THREADS) f32_rows_kernel(const float* __res
 }
 
 template <int WK>
-static void f32_rows_go(cudaStream_t st, const GemmProblem& p, int max_rows, bool ahead) {
+static void f32_rows_go(cudaStream_t st, const GemmProblem& p, int max_rows, bool ahead, bool below) {
   constexpr int FT = FR_F * (FR_THREADS / 32 / WK);
   const dim3 grid(cdiv(p.N, FT), cdiv(max_rows, FR_R));
 #define GO(KIND)                                                                                                  \
   launch_k(f32_rows_kernel<WK, KIND>, grid, FR_THREADS, 0, st, (const float*)p.A, p.lda, (const float*)p.B, p.ldb, \
-           p.rows, p.N, p.K, p.epi, ahead ? 1 : 0)
+           p.rows, p.N, p.K, p.epi, ahead ? 1 : 0, below ? 1 : 0)
   switch (p.epi.kind) {
     case EPI_F32: GO(EPI_F32); break;
     case EPI_ACT: GO(EPI_ACT); break;
@@ -229,31 +248,45 @@ static void f32_rows_go(cudaStream_t st, const GemmProblem& p, int max_rows, boo
 #undef GO
 }
 
-bool gemm_f32_rows(cudaStream_t st, const GemmProblem& p, int max_rows, bool ahead) {
-  if (max_rows < 1 || max_rows > F32_ROWS_MAX || p.N < 1 || p.K < 1) return false;
-  if ((p.K | p.lda | p.ldb) % 4 || (((uintptr_t)p.A | (uintptr_t)p.B) & 15)) return false;
-  if (p.epi.kind < EPI_F32 || p.epi.kind > EPI_KV) return false;
-  if ((p.epi.kind == EPI_SWIGLU || p.epi.kind >= EPI_QKV) && p.N % 32) return false;
+F32Rows gemm_f32_rows(cudaStream_t st, const GemmProblem& p, int max_rows, bool ahead) {
+  if (max_rows < 1 || max_rows > F32_ROWS_MAX || p.N < 1 || p.K < 1) return F32_ROWS_NONE;
+  if ((p.K | p.lda | p.ldb) % 4 || (((uintptr_t)p.A | (uintptr_t)p.B) & 15)) return F32_ROWS_NONE;
+  if (p.epi.kind < EPI_F32 || p.epi.kind > EPI_KV) return F32_ROWS_NONE;
+  if ((p.epi.kind == EPI_SWIGLU || p.epi.kind >= EPI_QKV) && p.N % 32) return F32_ROWS_NONE;
+  // Every count up to max_rows (within 64 rows the largest decides: the tiles' time stands still), or only the count itself
+  // where the host knows it. Otherwise the live count decides on the device: both kernels are launched, and the one whose count
+  // it is not leaves at once (2 to 20 us on products of 0.5 ms and more). The weights are then not read ahead.
+  bool all = f32_rows_win(max_rows, p.N, p.K);
+  if (!p.rows.begin && !p.rows.end) {
+    if (!all) return F32_ROWS_NONE;
+  } else {
+    for (int r = 64; r < max_rows; r += 64) all = all && f32_rows_win(r, p.N, p.K);
+  }
+  int most = max_rows;
+  while (most > 1 && !f32_rows_win(most, p.N, p.K)) --most;
   // K slices of 512 over 1, 2 or 4 warps
-  if (p.K <= FR_KC) f32_rows_go<1>(st, p, max_rows, ahead);
-  else if (p.K <= 2 * FR_KC) f32_rows_go<2>(st, p, max_rows, ahead);
-  else f32_rows_go<4>(st, p, max_rows, ahead);
-  return true;
+  if (p.K <= FR_KC) f32_rows_go<1>(st, p, most, ahead && all, !all);
+  else if (p.K <= 2 * FR_KC) f32_rows_go<2>(st, p, most, ahead && all, !all);
+  else f32_rows_go<4>(st, p, most, ahead && all, !all);
+  return all ? F32_ROWS_ALL : F32_ROWS_SOME;
 }
 
-void launch_gemm_simt(cudaStream_t st, int dt, const GemmProblem& p, int max_rows, float* scratch) {
+void launch_gemm_simt(cudaStream_t st, int dt, const GemmProblem& p, int max_rows, float* scratch, bool above) {
   if (max_rows <= 0) return;
   dim3 grid(cdiv(p.N, 64), cdiv(max_rows, 64));
+  const int up = above ? 1 : 0;
   if (dt == 1) {
     launch_k(gemm_simt_kernel<bf16>, grid, 256, 0, st, (const bf16*)p.A, p.lda, (const bf16*)p.B, p.ldb, p.rows, p.N, p.K,
-                                                 scratch, p.N);
-    launch_k(epilogue_kernel<bf16>, max_rows, 64, 0, st, p.epi, scratch, p.N, p.rows, p.N);
+                                                 scratch, p.N, up);
+    launch_k(epilogue_kernel<bf16>, max_rows, 64, 0, st, p.epi, scratch, p.N, p.rows, p.N, up, p.K);
   } else {
     launch_k(gemm_simt_kernel<float>, grid, 256, 0, st, (const float*)p.A, p.lda, (const float*)p.B, p.ldb, p.rows, p.N,
-                                                  p.K, scratch, p.N);
-    launch_k(epilogue_kernel<float>, max_rows, 64, 0, st, p.epi, scratch, p.N, p.rows, p.N);
+                                                  p.K, scratch, p.N, up);
+    launch_k(epilogue_kernel<float>, max_rows, 64, 0, st, p.epi, scratch, p.N, p.rows, p.N, up, p.K);
   }
 }
+
+extern "C" __attribute__((visibility("default"))) int adept_debug_f32_rows_win(int M, int N, int K) { return f32_rows_win(M, N, K); }
 
 ADEPT_KTRACE_ATTACH(simt)
 

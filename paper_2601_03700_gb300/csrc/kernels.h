@@ -117,11 +117,14 @@ void launch_tile_weight(cudaStream_t st, const void* src, int N, int K, int ld, 
 void launch_read_kv(cudaStream_t st, int dt, KVCacheView c, int layer0, int seq, int pos0, int n_pos, void* ko,
                     void* vo);
 
-// GEMMs.  SIMT path: C = A B^T into fp32 scratch, then the epilogue kernel.
-void launch_gemm_simt(cudaStream_t st, int dt, const GemmProblem& p, int max_rows, float* scratch);
+// GEMMs.  SIMT path: C = A B^T into fp32 scratch, then the epilogue kernel.  above: only where the live row count is not
+// gemm_f32_rows'.
+void launch_gemm_simt(cudaStream_t st, int dt, const GemmProblem& p, int max_rows, float* scratch, bool above = false);
 // fp32 problem of few rows in one launch (no scratch); ahead: B is a weight that no kernel still
-// running may write, read before the dependency wait.  False when the shape is not taken.
-bool gemm_f32_rows(cudaStream_t st, const GemmProblem& p, int max_rows, bool ahead);
+// running may write, read before the dependency wait.  NONE: not taken, nothing launched.  SOME: it takes some live row
+// counts, and launch_gemm_simt with `above` has to follow for the others.
+enum F32Rows { F32_ROWS_NONE, F32_ROWS_SOME, F32_ROWS_ALL };
+F32Rows gemm_f32_rows(cudaStream_t st, const GemmProblem& p, int max_rows, bool ahead);
 // Attention of the active query rows over the paged cache of one layer.
 // decode_keys > 0 (generation step, one query row per sequence): split-KV kernel over at
 // most decode_keys keys, using ws (>= rows * heads * ATTN_MAX_SPLIT * (head_dim + 2) floats)

@@ -493,10 +493,10 @@ static void gemm(adept_model* m, cudaStream_t st, const GemmProblem* probs, int 
   {
     for (int i = 0; i < n_probs; ++i) {
       // (a training product's second operand may be the preceding kernel's output)
-      if (m->dt == ADEPT_DTYPE_F32 && gemm_f32_rows(st, probs[i], max_rows[i], cls != ADEPT_PROF_GEMM_TRAIN)) {
-        m->launches += 1;
-        continue;
-      }
+      F32Rows taken = F32_ROWS_NONE;
+      if (m->dt == ADEPT_DTYPE_F32) taken = gemm_f32_rows(st, probs[i], max_rows[i], cls != ADEPT_PROF_GEMM_TRAIN);
+      if (taken != F32_ROWS_NONE) m->launches += 1;
+      if (taken == F32_ROWS_ALL) continue;
       if (!ensure_scratch(m, (size_t)max_rows[i] * probs[i].N)) {
         cudaStreamSynchronize(st);
         if (!ensure_scratch(m, (size_t)max_rows[i] * probs[i].N)) {   // the call returns OOM
@@ -504,7 +504,7 @@ static void gemm(adept_model* m, cudaStream_t st, const GemmProblem* probs, int 
           continue;
         }
       }
-      launch_gemm_simt(st, m->dt, probs[i], max_rows[i], m->scratch);
+      launch_gemm_simt(st, m->dt, probs[i], max_rows[i], m->scratch, taken == F32_ROWS_SOME);
       m->launches += 2;
     }
   }

@@ -35,3 +35,18 @@ def test_f32_rows_match_oracle(family, head_dim, B, P):
         compare_decode(pair, cache, ores.next_token, 3, 0.9, steps)
         pair.compare_cache(cache, B, P + 3)
     pair.close()
+
+
+@pytest.mark.parametrize("family,P", [(synth.LLAMA, 110), (synth.LLAMA, 111), (synth.LLAMA, 139), (synth.LLAMA, 250),
+                                      (synth.GPT2, 250)])
+def test_live_counts_on_both_sides_of_the_rule(family, P):
+    """Wide products (16384 outputs of K 520: the rows kernel up to 110 rows and from 129 to 138, the tiles at the other
+    counts; 8192 of the mapper up to 220), with live counts that fall from layer to layer across the line."""
+    cfg = synth.ModelConfig(family=family, n_layers=6, d_model=520, n_heads=4, head_dim=64,
+                            d_ffn=8192 if family == synth.LLAMA else 16384, vocab=517, max_pos=256, dtype="f32",
+                            hsm_m1=520, hsm_m2=8192, max_batch=1, max_seq=P, max_pass_tokens=P, block_shuffle_seed=3)
+    pair = Pair(cfg, weights=synth.make_weights(cfg, seed=130, std=0.03, device="cuda"))
+    tokens = synth.make_tokens(131, 1, P, 517).numpy()
+    compare_prefill(pair, tokens, 0.9, synth.forced_exits_uniform(132 + P, P, 2, 6).numpy().reshape(1, P))
+    compare_prefill(pair, tokens, -2.0)      # every token leaves at layer 2: all rows to the mapper, none after it
+    pair.close()
