@@ -1052,12 +1052,17 @@ void launch_attention(cudaStream_t st, int dt, const void* q, int ld_q, void* ou
     }
     return;
   }
-  if (dt == 1)
+  if (dt == 1) {
+    // After the paired GEMM (more than 128 rows) without an early start: a pair's CTA leaves an SM registers for one CTA of
+    // this kernel, an SM without one holds six, so CTAs that started beside it crowded the SMs that had none (512 rows of
+    // 8 heads of 32, 4 layers: 1.73 ms, 1.09 so; the start that is given up costs 2 us a layer).
+    PdlScope balanced(g_pdl && max_rows <= 128);
     attn_dispatch<bf16>(st, q, ld_q, out, ld_out, rows, max_rows, row_tok, tok_seq, tok_pos, seq_len, cache, layer0,
                         n_heads, causal);
-  else
+  } else {
     attn_dispatch<float>(st, q, ld_q, out, ld_out, rows, max_rows, row_tok, tok_seq, tok_pos, seq_len, cache, layer0,
                          n_heads, causal);
+  }
 }
 
 ADEPT_KTRACE_ATTACH(attention)
