@@ -40,6 +40,17 @@ def test_pair_gemm_prompt_matches_oracle(family, B, P):
     pair.close()
 
 
+@pytest.mark.parametrize("family", [synth.LLAMA, synth.GPT2])
+def test_pair_gemm_heads_of_32_match_oracle(family):
+    """One head per 32-column chunk: queries, keys (their rotary halves of 16) and values of the cache epilogue."""
+    pair = Pair(config(family, 1, 141, n_heads=10, n_kv_heads=5, head_dim=32), seed=126)
+    tokens = synth.make_tokens(127, 1, 141, 1003).numpy()
+    forced = synth.forced_exits_uniform(128, 141, 2, 5).numpy().reshape(1, 141)
+    _, cache, _ = compare_prefill(pair, tokens, 0.9, forced)
+    pair.compare_cache(cache, 1, 141)
+    pair.close()
+
+
 @pytest.mark.parametrize("n", [129, 300])
 def test_pair_gemm_grouped_fill_matches_oracle(n):
     cfg = config(synth.LLAMA, 1, 300, n_layers=9)

@@ -171,10 +171,10 @@ def test_synth_generator_cpu_and_cuda_agree():
 
 
 def test_prompt_pass_mapper_split_by_live_rows():
-    """The prompt pass's mapper products split by the device-side exit count (narrow tiles up
-    to the split bound, the bound's tiles above it): 600 tokens with 300 leaving at layer 2 and
-    100 at layers 3 and 4 take both launches of each split product (a D = 512 model with
-    mapper widths 2048 / 4096 so that the bound's tiles are wide enough to split)."""
+    """The prompt pass's mapper products at device-side exit counts near and far below their
+    bound: 600 tokens with 300 leaving at layer 2 and 100 at layers 3 and 4 (the paired tiles
+    take their width from the count; a D = 512 model with mapper widths 2048 / 4096, so that
+    the counts lie on both sides of a change of width)."""
     cfg = small(synth.GPT2, n_layers=6, d_model=512, n_heads=8, head_dim=64, d_ffn=1024, hsm_m1=2048, hsm_m2=4096,
                 max_seq=160, max_pos=160)
     pair = Pair(cfg, seed=12, std=0.04)

@@ -1,5 +1,5 @@
 """The last launch of a generation step: greedy tokens (the first of equal logits) and the copies of logits, exits and
-similarities, for vocabularies in one part and in many, over repeated steps and with outputs left out."""
+similarities, for vocabularies in one part and in many, over repeated steps and with outputs left out; logits that are NaN."""
 import pytest
 import torch
 
@@ -32,3 +32,26 @@ def test_step_outputs(vocab, batch):
         tok = nx.clone()
     m.check()
     m.close()
+
+
+@pytest.mark.parametrize("vocab", [1000, 4097])
+def test_nan_logits_are_never_the_token(vocab):
+    """A NaN logit is passed over, at a part's first and last column too; a row of nothing else gives token 0."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    cfg = synth.ModelConfig(family=synth.LLAMA, n_layers=3, d_model=128, n_heads=2, head_dim=64, d_ffn=256, vocab=vocab,
+                            dtype="bf16", hsm_m1=256, hsm_m2=512, max_batch=3, max_seq=32, max_pass_tokens=12)
+    W = synth.make_weights(cfg, seed=142, device="cuda")
+    tok = synth.make_tokens(143, 3, 4, vocab).cuda()
+    for bad in ([0, 129, vocab // 2, vocab - 1], list(range(vocab))):
+        head = W["lm_head"].clone()
+        head[bad] = float("nan")
+        m = adept.Model(cfg, {**W, "lm_head": head})
+        nx = m.prefill(tok, 0.9)[2]
+        for _ in range(3):   # launched directly, captured, replayed
+            _, lg, nx, _ = m.decode_step(nx.clone(), 0.9)
+            assert torch.isnan(lg[:, bad]).all() and int(torch.isnan(lg).sum()) == 3 * len(bad)
+            lg = lg.masked_fill(torch.isnan(lg), float("-inf"))
+            assert torch.equal(nx.long(), (lg == lg.max(dim=1, keepdim=True).values).int().argmax(dim=1))
+        m.check()
+        m.close()

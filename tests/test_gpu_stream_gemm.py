@@ -5,8 +5,8 @@ The model is sized so that the wide GEMMs of a generation step (at least 8 MB of
 (QKV 9216 outputs), SwiGLU 5504 (gate/up 11008 outputs; K = 5504 of the down projection ends in
 a half k-block), the 36 D^2 mapper (FC2 has 16384 outputs), a 9000-token vocabulary (the head's
 last 32-feature tile is ragged) and the grouped fills (6144 outputs per layer); the narrower
-products take the cluster K-split kernel.  Batches of 1, 5 and 12 sequences cover one and two 8-token
-blocks of the A operand.  Generation steps (forced exits through every layer, the mapper,
+products take the cluster K-split kernel.  Batches of 1 and 5 sequences take these kernels, one of
+12 the weight-streaming tcgen05 kernel (9 rows and more).  Generation steps (forced exits through every layer, the mapper,
 the grouped skipped-layer fill and the head) are compared with the oracle, with the cluster
 K-split kernel, and with themselves run again (the split tiles are summed in a fixed order, so
 the results are bit-identical); skipped-layer fills of 1 to 16 tokens through
@@ -112,8 +112,8 @@ def test_tile_contiguous_weights_give_identical_results(B):
 
 
 def test_stream_gemm_small_fills_match_oracle():
-    """adept_skip_kv_fill of 1, 3, 8, 9 and 16 tokens (the grouped stream-K launch over the
-    layers that have rows; 9-16 tokens use two 8-token blocks) against the oracle."""
+    """adept_skip_kv_fill of 1, 3 and 8 tokens (the grouped stream-K launch over the layers that
+    have rows) and of 9 and 16 (the weight-streaming tcgen05 kernel) against the oracle."""
     cfg = _cfg(4)
     W = synth.make_weights(cfg, seed=46, device="cuda")
     pair = Pair(cfg, weights=W)

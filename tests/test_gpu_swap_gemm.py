@@ -52,6 +52,19 @@ def test_swap_gemm_generation_matches_oracle(family, B):
     pair.close()
 
 
+@pytest.mark.parametrize("family", [synth.LLAMA, synth.GPT2])
+@pytest.mark.parametrize("B,P", [(9, 1), (1, 45)])
+def test_swap_gemm_heads_of_32_match_oracle(family, B, P):
+    """One head per 32-feature cell: queries, keys (their rotary halves of 16) and values of the cache epilogue."""
+    pair = Pair(config(family, B, P, n_heads=10, n_kv_heads=5, head_dim=32), seed=103)
+    tokens = synth.make_tokens(104, B, P, 1003).numpy()
+    forced = synth.forced_exits_uniform(105, B * P, 2, 5).numpy().reshape(B, P)
+    ores, cache, _ = compare_prefill(pair, tokens, 0.9, forced)
+    compare_decode(pair, cache, ores.next_token, 2, 0.9, synth.forced_exits_uniform(106, 2 * B, 2, 5).numpy().reshape(2, B))
+    pair.compare_cache(cache, B, P + 2)
+    pair.close()
+
+
 @pytest.mark.parametrize("n", [9, 33, 128])
 def test_swap_gemm_grouped_fill_matches_oracle(n):
     cfg = config(synth.LLAMA, 1, 128, n_layers=9)
@@ -83,3 +96,29 @@ def test_swap_gemm_repeats_bit_for_bit():
         assert torch.equal(first, m.prefill(tok, 0.9, fz)[1])
     m.check()
     m.close()
+
+
+def test_waits_running_out_at_any_point_leave_the_clusters_whole():
+    """Limits from a few cycles to a few microseconds stop the CTAs of a cluster at different k-blocks (tiles split over up to
+    8 CTAs, their rings deeper than a CTA's share and shallower): every pass ends, says so in its status, and the next one is
+    right."""
+    cfg = config(synth.LLAMA, 2, 30, n_layers=3, d_model=1024, n_heads=16, d_ffn=4096, hsm_m1=2048, hsm_m2=4096)
+    pair = Pair(cfg, weights=synth.make_weights(cfg, seed=107, device="cuda"))
+    tokens = synth.make_tokens(108, 2, 30, 1003).numpy()
+    forced = synth.forced_exits_uniform(109, 60, 2, 3).numpy().reshape(2, 30)
+    dev = lambda x: torch.as_tensor(x).cuda()  # noqa: E731
+    stopped = 0
+    for limit in (1, 32, 200, 500, 1000, 1500, 2000, 3000, 5000, 10000):
+        adept.adept_set_wait_limit(limit)
+        try:
+            pair.gm.prefill(dev(tokens), 0.9, dev(forced))
+            try:
+                pair.gm.check()
+            except adept.AdeptError as e:
+                assert e.status == 5, str(e)
+                stopped += 1
+        finally:
+            adept.adept_set_wait_limit(0)
+    assert stopped >= 2
+    compare_prefill(pair, tokens, 0.9, forced)
+    pair.close()
