@@ -407,7 +407,8 @@ struct GemmProblem {
   int K;
   Epi epi;
   // rows on the device that are usually far below their bound (the prompt pass's exiting
-  // rows): the tensor-core launcher may split the problem by the live count
+  // rows), often none: nothing of the problem is read ahead of their count, and the one-CTA
+  // tensor-core launcher may split the problem by it
   int split_live = 0;
   // Optional tile-contiguous copy of B for the weight-streaming kernels (NULL: none): 16 KB
   // units, one per (32-row tile, 256-k block), tile-major, each laid out as the kernels' shared-

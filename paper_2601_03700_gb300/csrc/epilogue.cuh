@@ -60,7 +60,9 @@ __device__ __forceinline__ EpiRow epi_row(const Epi& e, int ra) {
   return r;
 }
 
-// One pair turned by (cos, sin), its operations fixed so that every kernel rounds alike.
+// One pair turned by (cos, sin), its operations fixed so that the tcgen05 kernels (tiled, paired, streaming), which share
+// products of one shape, round alike. The mma.sync and fp32 kernels leave the contraction to the compiler; their sums are
+// in another order anyway.
 __device__ __forceinline__ float2 rope_turn(float x1, float x2, float co, float si) {
   return make_float2(fmaf(x1, co, -__fmul_rn(x2, si)), fmaf(x2, co, __fmul_rn(x1, si)));
 }

@@ -11,16 +11,16 @@ namespace adept {
 
 // Whether f32_rows_kernel takes M rows of an N x K product, and not the 64 x 64 tiles.
 //
-// The rows kernel reads every weight again for each 8 rows and takes M N K / 6e12 s (K of up to 512, where a warp has one slice
-// of K, and above 8192, where a row's pieces leave L1 between features: M N K / 3.3e12 s); the tiles take 0.18 us per element of K
-// while they find a place on the SMs at once, then as many times more as there are tiles (a ninth of an SM each). Both
-// sides measured over 31 (N, K) from 256 x 256 to 32768 x 8192 and up to 256 rows: the better kernel is chosen in all but a
-// few places near the line, and there it is within 13 %. Bounds of 64 and 128 rows, rows kernel / tiles in us:
-// 4096 x 4096 197 / 738 and 370 / 715; 12288 x 4096 566 / 887 and 1118 / 989; 8192 x 16384 2499 / 3209 and 4994 / 3172;
-// 32768 x 8192 3006 / 2081 and 5641 / 3634. Prompt of 256 rows, D = 4096, FFN 11008, 4 layers, mapper 8192 / 16384: 37.1 ms on
-// the tiles alone, 44.9 on the rows kernel alone, 29.0 so. Up to 256 rows, as prompt passes of a model of D = 1024 (4 layers, mapper
-// 4096 / 8192), all rows to full depth, take 1.15 / 2.24 / 4.43 / 9.20 ms at 64 / 128 / 256 / 512 rows here and
-// 4.59 / 4.68 / 5.85 / 8.53 on the tiles.
+// The rows kernel reads every weight again for each 8 rows and takes M N K / 6e12 s (above K = 8192, where a row's pieces leave L1
+// between features, M N K / 3.6e12 s); the tiles take 0.18 us per element of K while they find a place on the SMs at once (about
+// 120 tiles), then 1 / 608 of that more per tile. Up to K = 512 the launches weigh on the rows kernel (M N K / 4.6e12 s), and
+// the tiles take 0.13 us. So the line is 1.1 or 0.6 million outputs for one turn of the tiles. Both sides measured over 29
+// (N, K) from 256 x 256 to 32768 x 8192 and up to 256 rows: the better kernel is chosen in all but a few places near the
+// line, and there it is within 13 %. At 64 and 128 rows, rows kernel / tiles in us: 4096 x 4096 197 / 738 and 370 / 715;
+// 12288 x 4096 566 / 887 and 1118 / 989; 8192 x 16384 2499 / 3209 and 4994 / 3172; 32768 x 8192 3006 / 2081 and 5641 / 3634.
+// Prompt of 256 rows, D = 4096, FFN 11008, 4 layers, mapper 8192 / 16384: 37.1 ms on the tiles alone, 44.9 on the rows
+// kernel alone, 29.0 so; D = 1024 (mapper 4096 / 8192) 8.84, 5.35 and 5.02. Above 256 rows the tiles: of D = 1024, 512 rows
+// took 8.53 ms on them and 9.20 on the rows kernel.
 constexpr int F32_ROWS_MAX = 256;
 __host__ __device__ inline bool f32_rows_win(int M, int N, int K) {
   if (M > F32_ROWS_MAX) return false;

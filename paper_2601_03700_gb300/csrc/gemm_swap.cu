@@ -65,7 +65,6 @@ struct SwParams {
   int tmem_cols;  // accumulator columns (nt rounded up to 32, then to a power of two)
   int stages;
   int splits;     // cluster size
-  int m_hi;
   int apart;      // the cells' exchange has shared memory of its own at off_cells (0: over the ring)
   int off_cells;
   int ahead;      // weights before the dependency wait (not where there may well be no rows)
@@ -115,7 +114,7 @@ __global__ void __launch_bounds__(SW_THREADS) gemm_swap_kernel(const __grid_cons
     // nothing is read ahead: without rows the launch ends here
     pdl_wait();
     const int m = g.rows.e() - g.rows.b();
-    if (m <= 0 || (p.m_hi > 0 && m > p.m_hi)) return;   // (the whole cluster)
+    if (m <= 0) return;   // (the whole cluster)
   }
   const int k_lo = (int)((long long)rank * g.nks / splits), n_st = (int)((long long)(rank + 1) * g.nks / splits) - k_lo;
 
@@ -150,7 +149,6 @@ __global__ void __launch_bounds__(SW_THREADS) gemm_swap_kernel(const __grid_cons
   if (threadIdx.x == 0) {
     const int b = g.rows.b();
     int M = max(0, g.rows.e() - b);
-    if (p.m_hi > 0 && M > p.m_hi) M = 0;   // another launch's
     if (M > nt) {                          // more rows than the launch was sized for
       atomicOr(p.err, ERRW_CONFIG);
       M = nt;
@@ -339,14 +337,13 @@ int sw_launch(cudaStream_t st, const SwParams<MAXG>& prm, int grid, size_t smem)
 }
 
 template <int KC, int MAXG>
-int sw_go(cudaStream_t st, const GemmProblem* probs, int n, int rows, unsigned* err, int m_hi) {
+int sw_go(cudaStream_t st, const GemmProblem* probs, int n, int rows, unsigned* err) {
   thread_local SwParams<MAXG> prm;   // one per host thread
   memset(&prm, 0, sizeof prm);
   prm.n_groups = n;
   prm.nt = cdiv(rows, 16) * 16;
   prm.tmem_cols = 32;
   while (prm.tmem_cols < prm.nt) prm.tmem_cols *= 2;
-  prm.m_hi = m_hi;
   prm.ahead = 1;
   prm.err = err;
   prm.span = g_span;
@@ -403,15 +400,14 @@ bool swap_gemm_supported(const GemmProblem& q, int max_rows) {
   return q.epi.kind >= EPI_F32 && q.epi.kind <= EPI_KV;
 }
 
-int swap_gemm(cudaStream_t st, const GemmProblem* probs, int n_probs, const int* max_rows, unsigned* err, int m_hi) {
+int swap_gemm(cudaStream_t st, const GemmProblem* probs, int n_probs, const int* max_rows, unsigned* err) {
   if (n_probs < 1 || n_probs > SW_MAXG) return -1;
   int rows = 0;
   for (int i = 0; i < n_probs; ++i) {
     const GemmProblem& q = probs[i];
-    const int r = m_hi > 0 ? std::min(m_hi, max_rows[i]) : max_rows[i];
-    if (!swap_gemm_supported(q, r) || q.epi.tile_stats) return -1;
+    if (!swap_gemm_supported(q, max_rows[i]) || q.epi.tile_stats) return -1;
     if (n_probs > 1 && q.epi.kind != EPI_QKV && q.epi.kind != EPI_KV) return -1;
-    rows = std::max(rows, r);
+    rows = std::max(rows, max_rows[i]);
   }
   if (!g_sw_sms) {
     int dev = 0;
@@ -421,10 +417,10 @@ int swap_gemm(cudaStream_t st, const GemmProblem* probs, int n_probs, const int*
   }
   // two k-chunks per stage (256 contiguous bytes of a weight row) while two stages and more fit
   if (rows <= 16)
-    return n_probs <= 2 ? sw_go<2, 2>(st, probs, n_probs, rows, err, m_hi)
-                        : sw_go<2, SW_MAXG>(st, probs, n_probs, rows, err, m_hi);
-  return n_probs <= 2 ? sw_go<1, 2>(st, probs, n_probs, rows, err, m_hi)
-                      : sw_go<1, SW_MAXG>(st, probs, n_probs, rows, err, m_hi);
+    return n_probs <= 2 ? sw_go<2, 2>(st, probs, n_probs, rows, err)
+                        : sw_go<2, SW_MAXG>(st, probs, n_probs, rows, err);
+  return n_probs <= 2 ? sw_go<1, 2>(st, probs, n_probs, rows, err)
+                      : sw_go<1, SW_MAXG>(st, probs, n_probs, rows, err);
 }
 
 ADEPT_KTRACE_ATTACH(sw)

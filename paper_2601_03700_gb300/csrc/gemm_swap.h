@@ -12,11 +12,10 @@ constexpr int SW_MAXG = 32;        // problems of a grouped launch
 bool swap_gemm_supported(const GemmProblem& p, int max_rows);
 
 // Enqueues the problems (rows on the device, at most max_rows[i] <= SW_MAX_ROWS each) in one
-// launch.  m_hi > 0: a problem whose live count is above m_hi is left out (another launch takes
-// it).  Returns 1, or -1 when a shape is not taken (nothing launched): more than SW_MAX_ROWS
+// launch.  Returns 1, or -1 when a shape is not taken (nothing launched): more than SW_MAX_ROWS
 // rows, K not a multiple of 64, unaligned operands, or epilogue kinds that do not
 // share a launch (only EPI_QKV and EPI_KV do).
-int swap_gemm(cudaStream_t st, const GemmProblem* probs, int n_probs, const int* max_rows, unsigned* err, int m_hi = 0);
+int swap_gemm(cudaStream_t st, const GemmProblem* probs, int n_probs, const int* max_rows, unsigned* err);
 
 cudaError_t set_wait_limit_sw(long long cycles);
 

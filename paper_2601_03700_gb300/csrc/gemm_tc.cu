@@ -679,8 +679,9 @@ static int launch_grouped(cudaStream_t st, const GemmProblem* probs, int n_probs
   return launch_prepared(st, L);
 }
 
-// One problem whose live row count is on the device and usually far below its bound (the
-// prompt pass's exiting rows, flagged split_live): the host knows only the bound, whose tile
+// Where the paired kernel (gemm_pair.cu, which takes its tile width from the live count) cannot be launched: one problem
+// whose live row count is on the device and usually far below its bound (the prompt pass's exiting rows, flagged
+// split_live).  The host knows only the bound, whose tile
 // width can leave most SMs idle for the live count.  Two launches then share the problem: one
 // with the next narrower tiles for live counts up to m_split rows, the most row tiles that
 // width still fits in one wave (there each CTA loads (128 + BN) x K per tile instead of

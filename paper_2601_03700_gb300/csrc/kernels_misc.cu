@@ -3,6 +3,7 @@
 #define ADEPT_TU_ID 3
 #include "common.cuh"
 #include "kernels.h"
+#include "row_group.cuh"
 
 #include <math.h>
 
@@ -129,14 +130,6 @@ static int hsm_grid(int max_rows, int threads) { return row_grid(max_rows, 2048 
 // pass over memory: each row's s_i, inertia and s_{i-1} are read once into registers (a
 // row per 512 >> rshift threads), the decision and compaction run on the reduced sums,
 // and the moves are written from the registers.
-__device__ __forceinline__ void put_row4(float* o, int v, float4 a) { reinterpret_cast<float4*>(o)[v] = a; }
-__device__ __forceinline__ void put_row4(bf16* o, int v, float4 a) {
-  const __nv_bfloat162 lo = __floats2bfloat162_rn(a.x, a.y), hi = __floats2bfloat162_rn(a.z, a.w);
-  uint2 u;
-  u.x = *reinterpret_cast<const uint32_t*>(&lo);
-  u.y = *reinterpret_cast<const uint32_t*>(&hi);
-  reinterpret_cast<uint2*>(o)[v] = u;
-}
 constexpr int EXD_THREADS = 512;
 constexpr int EXD_V = 4;   // most float4 per thread per row vector
 // V: float4 per thread per row vector, the fewest that cover a row (the kernel runs cold in
@@ -301,7 +294,7 @@ __global__ void __launch_bounds__(EXD_THREADS)
         const int v = sub + j * tpr;
         if (v < D4) {
           const float4 a = xs[j];
-          put_row4(o, v, make_float4((a.x - m0) * rs, (a.y - m0) * rs, (a.z - m0) * rs, (a.w - m0) * rs));
+          put4(o, v, make_float4((a.x - m0) * rs, (a.y - m0) * rs, (a.z - m0) * rs, (a.w - m0) * rs));
         }
       }
     }

@@ -128,7 +128,7 @@ struct adept_model {
   // pass workspaces (T_max rows)
   int T_max = 0;
   float *X_in[2] = {nullptr, nullptr}, *X_out = nullptr, *I[2] = {nullptr, nullptr};
-  int *row_tok[2] = {nullptr, nullptr}, *tok_seq = nullptr, *tok_pos = nullptr, *flag = nullptr, *dst = nullptr;
+  int *row_tok[2] = {nullptr, nullptr}, *tok_seq = nullptr, *tok_pos = nullptr, *flag = nullptr;
   float* inv_norm = nullptr;
   float *hsm_s = nullptr, *hsm_prev = nullptr, *hsm_I = nullptr;
   int* exit_tok = nullptr;
@@ -865,7 +865,6 @@ static adept_status alloc_runtime(adept_model* m) {
   TRY(dalloc_t(m, &m->tok_seq, T));
   TRY(dalloc_t(m, &m->tok_pos, T));
   TRY(dalloc_t(m, &m->flag, T));
-  TRY(dalloc_t(m, &m->dst, T));
   TRY(dalloc_t(m, &m->inv_norm, T));
   TRY(dalloc_t(m, &m->hsm_s, TD));
   TRY(dalloc_t(m, &m->hsm_prev, TD));
