@@ -340,6 +340,7 @@ static void prof_end(adept_model* m, int cls, cudaStream_t st, cudaEvent_t b, do
 static bool ensure_scratch(adept_model* m, size_t elems) {
   if (elems <= m->scratch_elems) return true;
   if (m->scratch) {
+    drop_graphs(m);   // captured steps hold its address
     cudaFree(m->scratch);
     m->allocs.erase(std::remove(m->allocs.begin(), m->allocs.end(), (void*)m->scratch), m->allocs.end());
     m->scratch = nullptr;

@@ -156,3 +156,30 @@ def test_refused_step_graph_leaves_the_sequences_as_they_were(dtype):
     compare_decode(pair, cache, tok, 3, 0.9, steps[1:])
     pair.compare_cache(cache, 3, 9)
     pair.close()
+
+
+def test_captured_step_does_not_outlive_the_scratch_it_holds():
+    """Training workspaces that grow the scratch of the SIMT products give its old memory back: the generation step captured
+    on it is captured anew (refused here by the allocation hook, to see that it is), and the steps match the oracle."""
+    cfg = synth.ModelConfig(family=synth.LLAMA, n_layers=3, d_model=128, n_heads=2, head_dim=64, d_ffn=256, vocab=500,
+                            dtype="bf16", max_batch=2, max_seq=32, hsm_m1=256, hsm_m2=512, max_pass_tokens=8,
+                            block_shuffle_seed=4)
+    pair = Pair(cfg, seed=56)
+    adept.adept_set_option(pair.gm.h, adept.OPT_GEMM_SIMT, 1)
+    tokens = synth.make_tokens(56, 2, 4, cfg.vocab).numpy()
+    ores, cache, _ = compare_prefill(pair, tokens, 0.9, np.full((2, 4), 3))
+    steps = np.array([[2, 3]] * 6)
+    compare_decode(pair, cache, ores.next_token, 3, 0.9, steps[:3])   # launched, captured, replayed
+    adept.adept_hsm_train_init(pair.gm.h, 2000)
+    compare_decode(pair, cache, ores.next_token, 1, 0.9, steps[3:4])
+    adept.adept_set_alloc_fail_after(0)
+    try:
+        with pytest.raises(adept.AdeptError) as ei:
+            pair.gm.decode_step(torch.as_tensor(ores.next_token, dtype=torch.int32).cuda(), 0.9,
+                                torch.as_tensor(steps[4], dtype=torch.int32).cuda())
+        assert ei.value.status == OOM
+    finally:
+        adept.adept_set_alloc_fail_after(-1)
+    compare_decode(pair, cache, ores.next_token, 2, 0.9, steps[4:])
+    pair.compare_cache(cache, 2, 10)
+    pair.close()
