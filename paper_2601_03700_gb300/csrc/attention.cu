@@ -13,12 +13,12 @@ namespace adept {
 
 // One warp per (query row, head); lanes own keys for the scores and head dimensions
 // for the value sum; online softmax over blocks of 32 keys.
-template <typename T, int DH>
+template <typename T, int DH, bool MASK>
 __global__ void __launch_bounds__(256) attn_warp_kernel(const T* __restrict__ q, int ld_q, T* __restrict__ out,
                                                         int ld_out, DevRange rows, const int* row_tok,
                                                         const int* tok_seq, const int* tok_pos, const int* seq_len,
                                                         KVCacheView cache, int layer0, int n_heads, int causal,
-                                                        float scale) {
+                                                        float scale, const int* key_exit, int kp_len) {
   PDL_ENTRY();
   __shared__ float qs[8][DH];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -43,7 +43,9 @@ __global__ void __launch_bounds__(256) attn_warp_kernel(const T* __restrict__ q,
   for (int kb = 0; kb < nk; kb += 32) {
     const int key = kb + lane;
     float s = -INFINITY;
-    if (key < nk) {
+    // (MASK: keys of tokens that left before this layer have no K/V here)
+    const bool there = key < nk && (!MASK || key_exit[seq * kp_len + key] > layer0);
+    if (there) {
       const T* kr = K + cache.offset(layer0, seq, key, kvh);
       float a = 0.f;
 #pragma unroll 8
@@ -51,7 +53,8 @@ __global__ void __launch_bounds__(256) attn_warp_kernel(const T* __restrict__ q,
       s = a;
     }
     const float mn = fmaxf(m, warp_max(s));
-    const float p = key < nk ? expf(s - mn) : 0.f;
+    const float p = there ? expf(s - mn) : 0.f;
+    const unsigned present = MASK ? __ballot_sync(0xffffffffu, there) : 0xffffffffu;
     const float corr = (m == -INFINITY) ? 0.f : expf(m - mn);
     l = l * corr + warp_sum(p);
 #pragma unroll
@@ -59,6 +62,7 @@ __global__ void __launch_bounds__(256) attn_warp_kernel(const T* __restrict__ q,
     const int nb = min(32, nk - kb);
     for (int kk = 0; kk < nb; ++kk) {
       const float pk = __shfl_sync(0xffffffffu, p, kk);
+      if (MASK && !(present >> kk & 1u)) continue;
       const T* vr = V + cache.offset(layer0, seq, kb + kk, kvh);
 #pragma unroll
       for (int j = 0; j < PER; ++j) acc[j] = fmaf(pk, to_f(vr[lane + 32 * j]), acc[j]);
@@ -440,19 +444,21 @@ __global__ void attn_decode_combine_kernel(DevRange rows, int n_heads, int n_spl
 template <typename T>
 static void attn_dispatch(cudaStream_t st, const void* q, int ld_q, void* out, int ld_out, DevRange rows,
                           int max_rows, const int* row_tok, const int* tok_seq, const int* tok_pos,
-                          const int* seq_len, KVCacheView cache, int layer0, int n_heads, int causal) {
+                          const int* seq_len, KVCacheView cache, int layer0, int n_heads, int causal,
+                          const int* key_exit, int kp_len) {
   const int dh = cache.head_dim;
   const float scale = 1.f / sqrtf((float)dh);
   const int grid = cdiv(max_rows * n_heads, 8);
-#define ATT_CASE(D)                                                                                         \
-  case D:                                                                                                   \
-    launch_k(attn_warp_kernel<T, D>, grid, 256, 0, st, (const T*)q, ld_q, (T*)out, ld_out, rows, row_tok, tok_seq, \
-                                                 tok_pos, seq_len, cache, layer0, n_heads, causal, scale);  \
-    break;
+#define ATT_CASE(D, MASK)                                                                                          \
+  launch_k(attn_warp_kernel<T, D, MASK>, grid, 256, 0, st, (const T*)q, ld_q, (T*)out, ld_out, rows, row_tok, tok_seq, \
+           tok_pos, seq_len, cache, layer0, n_heads, causal, scale, key_exit, kp_len)
   switch (dh) {
-    ATT_CASE(32)
-    ATT_CASE(64)
-    ATT_CASE(128)
+    case 32:   // (the key mask is bf16 encoders'; with heads of 64 and 128 they take the mma.sync kernel)
+      if (key_exit) ATT_CASE(32, true);
+      else ATT_CASE(32, false);
+      break;
+    case 64: ATT_CASE(64, false); break;
+    case 128: ATT_CASE(128, false); break;
     default:
       break;
   }
@@ -1058,10 +1064,10 @@ void launch_attention(cudaStream_t st, int dt, const void* q, int ld_q, void* ou
     // 8 heads of 32, 4 layers: 1.73 ms, 1.09 so; the start that is given up costs 2 us a layer).
     PdlScope balanced(g_pdl && max_rows <= 128);
     attn_dispatch<bf16>(st, q, ld_q, out, ld_out, rows, max_rows, row_tok, tok_seq, tok_pos, seq_len, cache, layer0,
-                        n_heads, causal);
+                        n_heads, causal, key_exit, kp_len);
   } else {
     attn_dispatch<float>(st, q, ld_q, out, ld_out, rows, max_rows, row_tok, tok_seq, tok_pos, seq_len, cache, layer0,
-                         n_heads, causal);
+                         n_heads, causal, key_exit, kp_len);
   }
 }
 

@@ -367,3 +367,17 @@ def test_encoder_stop_entirely_matches_oracle():
                 assert_rows_close(v[ok], cache.V[l - 1][b, :P][ok], pair.tol, f"V layer {l} seq {b}")
     adept.adept_set_option(pair.gm.h, adept.OPT_STOP_ENTIRELY, 0)
     pair.close()
+
+
+@pytest.mark.parametrize("B,P", [(3, 40), (1, 240)])
+def test_encoder_stop_entirely_with_heads_of_32(B, P):
+    """The key mask in the attention of heads of 32, keys in several blocks of 32, whole blocks of them gone."""
+    cfg = small(synth.BERT, n_layers=6, n_heads=8, n_kv_heads=4, head_dim=32, n_classes=2, max_pos=P, max_seq=P,
+                max_batch=B)
+    pair = Pair(cfg, seed=31)
+    tokens = synth.make_tokens(31, B, P, cfg.vocab).numpy()
+    mixed = synth.forced_exits_uniform(32, B * P, 2, 6).numpy().reshape(B, P)
+    blocks = np.where(np.arange(P)[None, :] // 32 % 2 == 0, 2, mixed)   # whole blocks gone after layer 2
+    for forced in (mixed, blocks):
+        compare_prefill(pair, tokens, 0.9, forced, check_cache=False, stop_entirely=True)
+    pair.close()
