@@ -1937,6 +1937,7 @@ adept_status adept_decode_step(adept_model* m, int batch, const int32_t* d_token
     TRY(body(st));
     m->dec_warm[batch] += 1;
   }
+  m->last_rows = batch;   // (a replayed step does not pass through run_pass)
   for (int b = 0; b < batch; ++b) m->h_seq_len[b] += 1;
   // outputs out of the staging buffers and the greedy tokens, one launch
   if (d_exit_layer_out || d_next_token_out || d_logits_out || d_sim_out) {

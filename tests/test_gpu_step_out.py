@@ -55,3 +55,20 @@ def test_nan_logits_are_never_the_token(vocab):
             assert torch.equal(nx.long(), (lg == lg.max(dim=1, keepdim=True).values).int().argmax(dim=1))
         m.check()
         m.close()
+
+
+def test_final_states_of_a_replayed_step():
+    """The rows that may be read after a step are that step's, also when it is replayed after steps of another batch."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    cfg = synth.ModelConfig(family=synth.GPT2, n_layers=3, d_model=128, n_heads=2, head_dim=64, d_ffn=256, vocab=500,
+                            max_pos=64, dtype="bf16", hsm_m1=256, hsm_m2=512, max_batch=5, max_seq=32, max_pass_tokens=20)
+    m = adept.Model(cfg, synth.make_weights(cfg, seed=144, device="cuda"))
+    m.prefill(synth.make_tokens(145, 5, 4, cfg.vocab).cuda(), 0.9)
+    for batch in (5, 5, 5, 2, 2, 5, 2, 5):   # each launched directly, captured, replayed
+        m.decode_step(torch.arange(batch, dtype=torch.int32, device="cuda"), 0.9)
+        assert torch.isfinite(m.final_states(batch)).all()
+        with pytest.raises(adept.AdeptError):
+            m.final_states(batch + 1)
+    m.check()
+    m.close()
