@@ -1928,8 +1928,8 @@ adept_status adept_decode_step(adept_model* m, int batch, const int32_t* d_token
     const cudaError_t e = cudaGraphLaunch(m->dec_graph[batch], st);
     if (e != cudaSuccess) {
       // the set-up has run and the step has not: the lengths as they were
-      cudaGetLastError();
       cudaMemcpyAsync(m->d_seq_len, m->h_seq_len.data(), batch * sizeof(int), cudaMemcpyHostToDevice, st);
+      cudaGetLastError();   // reported here; the next call starts clean
       return fail(m, ADEPT_ERR_CUDA, "graph launch failed: %s", cudaGetErrorString(e));
     }
     m->launches += m->graph_launches;
